@@ -71,6 +71,13 @@ struct RoundStats {
 // in-neighbours that did not change).
 constexpr double kTestDensity = 0.5;
 
+// Dense rounds of graphs of at least this many arcs stop a row once it can
+// gain nothing more (pull_dense). The stop waits for the row's signature and
+// the seeds' counts before the first gather: on 0.55 M arcs (s = 300) a dense
+// round took 33 us with it and 27 without, on 65 M arcs (s = 256) the last
+// two took 136 and 132 us instead of 446 and 422.
+constexpr int64_t kEarlyStopArcs = 1LL << 22;
+
 struct Params {
   int64_t n, m;
   const int64_t *row_ptr;  // in-CSR
@@ -134,6 +141,7 @@ struct Params {
   float dense_threshold;
   int32_t row_cap;      // rows of the device counts window
   int32_t test_changed; // test C_{t-1} before gathering an in-neighbour's delta
+  int32_t early_stop;   // dense rounds stop rows that can gain nothing more
   int32_t test_adapt;   // decide test_changed per round (ctrl->test, set by the post kernel)
   int32_t dense_tma;    // dense rounds are swept by k_pull_tma (launched before k_pull)
   int32_t push;         // sparse rounds push from the previous frontier (kModePush)

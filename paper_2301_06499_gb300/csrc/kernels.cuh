@@ -294,8 +294,9 @@ __device__ __forceinline__ void frontier_append(const Params &p, Ctrl *ctrl, int
 
 // Finishes one row piece after its deltas are ORed into acc (words
 // [c*CW, c*CW+CW) of the row): a row of one piece compares with X[v] and
-// writes Y[v] if it changed; a row cut into pieces ORs acc into Y[v] with
-// atomics and reports a change when its OR added a bit.
+// writes Y[v] if it changed; a row cut into pieces ORs the bits its signature
+// lacks (own; all of acc when the caller passes zeros) into Y[v] with atomics
+// and reports a change when its OR added a bit.
 template <int CW>
 __device__ __forceinline__ bool finish_piece(const Params &p, int32_t v, int c, bool whole,
                                              const uint64_t (&own)[CW],
@@ -312,13 +313,14 @@ __device__ __forceinline__ bool finish_piece(const Params &p, int32_t v, int c, 
     if (changed) store_words<CW>(p.Y + (size_t)v * Wp + c * CW, nw);
   } else {
 #pragma unroll
-    for (int k = 0; k < CW; ++k)
-      if (acc[k]) {
-        const unsigned long long old =
-            atomicOr(reinterpret_cast<unsigned long long *>(p.Y + (size_t)v * Wp + c * CW + k),
-                     (unsigned long long)acc[k]);
-        changed |= (old | acc[k]) != old;
+    for (int k = 0; k < CW; ++k) {
+      const unsigned long long gain = acc[k] & ~own[k];
+      if (gain) {
+        const unsigned long long old = atomicOr(
+            reinterpret_cast<unsigned long long *>(p.Y + (size_t)v * Wp + c * CW + k), gain);
+        changed |= (old | gain) != old;
       }
+    }
   }
   return changed;
 }
@@ -331,8 +333,9 @@ __device__ __forceinline__ bool finish_piece(const Params &p, int32_t v, int c, 
 // to each pass on its own, as if the passes ran one after another. Adds the
 // active passes of one row piece to words (and their seeds to seeds); a row
 // cut into pieces is counted once per pass, by the piece whose claim bit
-// for that pass is set first.
-template <int CW>
+// for that pass is set first. OWN: the caller holds the row's words in own
+// (else only for rows of one piece).
+template <int CW, bool OWN>
 __device__ __forceinline__ void count_pass_words(const Params &p, int32_t v, int c, bool whole,
                                                  const uint64_t (&own)[CW],
                                                  const uint64_t (&acc)[CW], uint32_t *Kw,
@@ -344,8 +347,9 @@ __device__ __forceinline__ void count_pass_words(const Params &p, int32_t v, int
     if (!whole && set_bit(Kw + (size_t)w * (size_t)p.nbm, v)) continue;
     const uint64_t vm = valid_mask(w, p.s);
     const uint64_t x =
-        whole ? own[k]
-              : __ldg(reinterpret_cast<const unsigned long long *>(p.X) + (size_t)v * p.Wp + w);
+        OWN || whole
+            ? own[k]
+            : __ldg(reinterpret_cast<const unsigned long long *>(p.X) + (size_t)v * p.Wp + w);
     if ((x | ~vm) != ~0ULL) {
       ++words;
       seeds += (uint32_t)__popcll(vm);
@@ -511,6 +515,28 @@ __device__ __forceinline__ void gm_add_chunk(const Params &p, const Ctrl *ctrl, 
               sum);
 }
 
+// Bits that can still travel in round t: seed i's only if it gained a pair in
+// round t-1 (its ball grows by one layer a round, so a round without a new
+// node ends it, and every delta of round t-1 holds bits of growing seeds
+// only). One 64-bit mask per signature word, for the whole block; the seeds'
+// counts of round t-1 are complete when round t starts. Rows of more words
+// than kAliveWords and packed batches use the seeds' valid bits instead.
+constexpr int kAliveWords = 8;
+
+__device__ __forceinline__ void alive_masks(const Params &p, const Ctrl *ctrl, int t,
+                                            uint64_t *alive) {
+  const int lane = threadIdx.x & 31;
+  const int prev = t - 1 - ctrl->row_base;  // < 0: the row left with the last window
+  const uint32_t *row = p.counts + (size_t)(prev < 0 ? 0 : prev) * (size_t)p.ncols;
+  for (int w = threadIdx.x >> 5; w < p.Wp; w += kBlock / 32) {
+    const int i = w * 64 + lane;
+    const unsigned lo = __ballot_sync(kFullMask, i < p.s && (prev < 0 || row[i] != 0u));
+    const unsigned hi = __ballot_sync(kFullMask, i + 32 < p.s && (prev < 0 || row[i + 32] != 0u));
+    if (lane == 0) alive[w] = ((uint64_t)hi << 32) | lo;
+  }
+  __syncthreads();
+}
+
 // Dense round over the sliced-ELL copy: a warp per chunk of 32 pieces, lane
 // l owns piece l; step k reads arc k of all 32 pieces in one coalesced load,
 // and the U deltas of a lane's U steps are gathered together. The sweep is
@@ -521,7 +547,19 @@ __device__ __forceinline__ void gm_add_chunk(const Params &p, const Ctrl *ctrl, 
 //    a chunk starts and its first U column indices when the chunk ends
 //    (before the frontier append), ahead of the saturation test: there the
 //    latency matters more than the reads wasted on saturated rows.
-template <int CW, bool PW>
+//
+// A lane stops at the arc where its row can gain nothing more: when every bit
+// that still travels (alive, or the seeds' valid bits) is in the row's
+// signature or in the deltas it has gathered. What is left is whether the row
+// is active at all (some in-neighbour changed; per pass for PW): a row that
+// could gain nothing to begin with tests its in-neighbours' changed bits and
+// stops at the first one set. This is Alg. 2's early break on all words of a
+// row at once. On R-MAT graphs the growing seeds' balls meet in the hubs, so
+// that the rounds after the largest need 1-4% of their arcs (simulated on
+// 2^21 nodes, 63.5 M arcs, s = 512: 2.7 M gathers instead of 63.5 M, then
+// 0.5 M instead of 56 M). EARLY = p.early_stop: graphs of at least
+// kEarlyStopArcs arcs; smaller ones are swept whole.
+template <int CW, bool PW, bool EARLY>
 __device__ __forceinline__ void pull_dense(const Params &p, Ctrl *ctrl, const uint64_t *Dprev,
                                            const uint32_t *Cprev, int32_t *F, uint32_t *Ccur,
                                            uint32_t *Kcur, uint32_t *Kwcur, int lane,
@@ -531,7 +569,8 @@ __device__ __forceinline__ void pull_dense(const Params &p, Ctrl *ctrl, const ui
                                            uint32_t &my_scan,
                                            uint32_t &my_gath,
                                            uint32_t &my_items,
-                                           uint32_t &my_rows, int32_t *stage, int &scnt) {
+                                           uint32_t &my_rows, int32_t *stage, int &scnt,
+                                           const uint64_t *alive) {
   constexpr int U = CW <= 2 ? PG_DENSE_UNROLL_NARROW : PG_DENSE_UNROLL_WIDE;
   const bool tc = test_changed_now(p, ctrl);
   constexpr bool kPrefetch = CW <= 2;
@@ -603,55 +642,87 @@ __device__ __forceinline__ void pull_dense(const Params &p, Ctrl *ctrl, const ui
     }
     bool row_changed = false, any_delta = false;
     uint32_t pw_words = 0, pw_seeds = 0;
+    const int sv = alive || !EARLY ? p.s : (act ? seeds_of(p, v) : 0);
     for (int ch = 0; ch < nch; ++ch) {
       uint64_t own[CW], acc[CW];
 #pragma unroll
       for (int k = 0; k < CW; ++k) own[k] = acc[k] = 0;
-      if (act && whole) load_words<CW>(own, p.X + (size_t)v * Wp + ch * CW);
+      if (act && (EARLY || whole)) load_words<CW>(own, p.X + (size_t)v * Wp + ch * CW);
+      // the row's open words: bits it may still gain, or (PW) a pass of it
+      // whose activity is not known yet
+      auto limit = [&](int k) {
+        return alive ? alive[ch * CW + k] : valid_mask(ch * CW + k, sv);
+      };
+      auto can_gain = [&]() {
+        uint64_t r = 0;
+#pragma unroll
+        for (int k = 0; k < CW; ++k) {
+          const uint64_t lim = limit(k);
+          r |= lim & ~(own[k] | acc[k]);
+          if (PW && !acc[k] && lim && (own[k] | ~valid_mask(ch * CW + k, p.s)) != ~0ULL) r |= 1ULL;
+        }
+        return r != 0ULL;
+      };
+      bool open = act && (!EARLY || can_gain());
+      bool need = EARLY ? open || (act && !PW && !any_delta) : act;  // else the lane is done
       int32_t u[U];
 #pragma unroll
       for (int q = 0; q < U; ++q)
-        u[q] = !act ? -1 : ch == 0 ? u0[q] : (q < len ? __ldg(cc + 32LL * q) : -1);
+        u[q] = !need ? -1 : ch == 0 ? u0[q] : (q < len ? __ldg(cc + 32LL * q) : -1);
       for (int k0 = 0; k0 < clen; k0 += U) {
+        if (EARLY && !__any_sync(kFullMask, need)) break;
         const bool more = kPipe && k0 + U < clen;  // warp-uniform
         int32_t un[U];
         if (!kPipe && k0 > 0) {
 #pragma unroll
           for (int q = 0; q < U; ++q)
-            u[q] = (act && k0 + q < len) ? __ldg(cc + 32LL * (k0 + q)) : -1;
+            u[q] = (need && k0 + q < len) ? __ldg(cc + 32LL * (k0 + q)) : -1;
         }
         if (more) {
 #pragma unroll
           for (int q = 0; q < U; ++q)
-            un[q] = (act && k0 + U + q < len) ? __ldg(cc + 32LL * (k0 + U + q)) : -1;
+            un[q] = (need && k0 + U + q < len) ? __ldg(cc + 32LL * (k0 + U + q)) : -1;
         }
-        if (tc) {
+        if (EARLY && need && ch == 0) my_scan += (uint32_t)max(0, min(U, len - k0));
+        if (open) {
+          if (tc) {
 #pragma unroll
-          for (int q = 0; q < U; ++q)
-            if (u[q] >= 0 && !test_bit(Cprev, u[q])) u[q] = -1;
-        }
-#pragma unroll
-        for (int q = 0; q < U; ++q)
-          if (u[q] >= 0) {
-            if (gather_ok(p, u[q], ch * CW + CW - 1))
-              or_words<CW>(acc, Dprev + (size_t)u[q] * Wp + ch * CW);
-            if (ch == 0) ++my_gath;
+            for (int q = 0; q < U; ++q)
+              if (u[q] >= 0 && !test_bit(Cprev, u[q])) u[q] = -1;
           }
+#pragma unroll
+          for (int q = 0; q < U; ++q)
+            if (u[q] >= 0) {
+              if (gather_ok(p, u[q], ch * CW + CW - 1))
+                or_words<CW>(acc, Dprev + (size_t)u[q] * Wp + ch * CW);
+              if (ch == 0) ++my_gath;
+            }
+          if (EARLY) {
+#pragma unroll
+            for (int k = 0; k < CW; ++k) any_delta |= acc[k] != 0ULL;
+            open = can_gain();
+          }
+        } else if (need) {  // only whether the row is active
+#pragma unroll
+          for (int q = 0; q < U; ++q)
+            if (u[q] >= 0 && gather_ok(p, u[q], 0)) any_delta |= test_bit(Cprev, u[q]);
+        }
+        if (EARLY) need = open || (need && !PW && !any_delta);
         if (more) {
 #pragma unroll
-          for (int q = 0; q < U; ++q) u[q] = un[q];
+          for (int q = 0; q < U; ++q) u[q] = need ? un[q] : -1;
         }
       }
 #pragma unroll
       for (int k = 0; k < CW; ++k) any_delta |= acc[k] != 0ULL;
       if constexpr (PW)
-        if (act) count_pass_words<CW>(p, v, ch, whole, own, acc, Kwcur, pw_words, pw_seeds);
+        if (act) count_pass_words<CW, EARLY>(p, v, ch, whole, own, acc, Kwcur, pw_words, pw_seeds);
       if (act) row_changed |= finish_piece<CW>(p, v, ch, whole, own, acc);
     }
     if (has_next) first_batch((int)(it_next.y & 0x7FFFFFFFULL), off_next);
     if (act) {
       ++my_items;
-      my_scan += (uint32_t)len;
+      if (!EARLY) my_scan += (uint32_t)len;
     }
     act = act && any_delta;  // no changed in-neighbour: not active in round t
     uint32_t gdeg = 0;       // this lane's m_active of the chunk
@@ -799,7 +870,7 @@ __device__ __forceinline__ void pull_sparse(const Params &p, Ctrl *ctrl, const R
         for (int k = 0; k < CW; ++k) acc[k] |= __shfl_xor_sync(kFullMask, acc[k], off);
       }
       if constexpr (PW)
-        if (act && gl == 0) count_pass_words<CW>(p, v, c, whole, own, acc, Kwcur, pw_words, pw_seeds);
+        if (act && gl == 0) count_pass_words<CW, false>(p, v, c, whole, own, acc, Kwcur, pw_words, pw_seeds);
       if (act && gl == 0) row_changed |= finish_piece<CW>(p, v, c, whole, own, acc);
     }
     if (PW && pw_words) {  // passes as words: m_active here, not at the claim
@@ -985,10 +1056,20 @@ __global__ void __launch_bounds__(kBlock, CW <= 4 ? PG_PULL_MIN_BLOCKS : PG_PULL
   int scnt = 0;
   // dense rounds sweep every row; mixed rounds (a packed batch) sweep the rows
   // of the graphs that chose a full sweep and take the others' work list
-  if ((mode == kModeDense && !p.dense_tma) || mode == kModeMixed)  // dense_tma: k_pull_tma
-    pull_dense<CW, PW>(p, ctrl, rb.Dprev, rb.Cprev, rb.F, rb.Ccur, rb.Kcur, rb.Kwcur, lane, warp,
-                       nwarps, my_mact, my_work, my_scan, my_gath, my_items, my_rows, stage,
-                       scnt);
+  if ((mode == kModeDense && !p.dense_tma) || mode == kModeMixed) {  // dense_tma: k_pull_tma
+    if (p.early_stop) {
+      __shared__ uint64_t s_alive[kAliveWords];
+      const bool use_alive = !p.node_graph && p.Wp <= kAliveWords;
+      if (use_alive) alive_masks(p, ctrl, t, s_alive);
+      pull_dense<CW, PW, true>(p, ctrl, rb.Dprev, rb.Cprev, rb.F, rb.Ccur, rb.Kcur, rb.Kwcur,
+                               lane, warp, nwarps, my_mact, my_work, my_scan, my_gath, my_items,
+                               my_rows, stage, scnt, use_alive ? s_alive : nullptr);
+    } else {
+      pull_dense<CW, PW, false>(p, ctrl, rb.Dprev, rb.Cprev, rb.F, rb.Ccur, rb.Kcur, rb.Kwcur,
+                                lane, warp, nwarps, my_mact, my_work, my_scan, my_gath, my_items,
+                                my_rows, stage, scnt, nullptr);
+    }
+  }
   if (mode == kModeSparse || mode == kModeMixed)
     pull_sparse<CW, G, PW>(p, ctrl, rb, lane, warp, nwarps, my_mact, my_work, my_scan, my_gath,
                            my_items, my_rows, stage, scnt);

@@ -1129,6 +1129,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   p.test_changed = cl.o.test_changed == 1 || cl.o.test_changed == 3 ||
                    (cl.o.test_changed == 0 && big);
   p.test_adapt = !p.gfsum && (cl.o.test_changed == 3 || (cl.o.test_changed == 0 && big));
+  p.early_stop = g->m >= kEarlyStopArcs;
   p.use_cond = 0;
   p.cond = 0ULL;
   p.iter_guard = cl.max_rounds + 2;

@@ -233,7 +233,7 @@ __global__ void __launch_bounds__(kBlock, 1)
     for (int k = 0; k < CW; ++k) any_delta |= acc[k] != 0ULL;
     uint32_t pw_words = 0, pw_seeds = 0;
     if constexpr (PW)
-      if (act) count_pass_words<CW>(p, v, 0, whole, own, acc, Kwcur, pw_words, pw_seeds);
+      if (act) count_pass_words<CW, false>(p, v, 0, whole, own, acc, Kwcur, pw_words, pw_seeds);
     const bool row_changed = act && finish_piece<CW>(p, v, 0, whole, own, acc);
     if (act) {
       ++my_items;

@@ -132,9 +132,13 @@ typedef struct {
                                exceed 64 MiB (n x words per row x 8 bytes),
                                else 2 (a packed batch: 1 instead of 3) */
   int32_t planes_per_pass;  /* PROPAGATE-S: seeds per pass, 1..64; 0 = 64 */
-  int32_t use_graphs;       /* 1: the round loop is one CUDA graph with a
-                               device-driven while node (no host round trip
-                               per round); 0: plain launches in batches */
+  int32_t use_graphs;       /* 1: the rounds follow each other on the device
+                               without a host round trip: for rows of up to 8
+                               words gathered whole (s <= 512, or up to 8
+                               passes as words) with sparse_push 0 one
+                               cooperative launch holds the whole round loop,
+                               otherwise a CUDA graph with a device-driven
+                               while node; 0: plain launches in batches */
   int32_t timing;           /* 1: record CUDA events around every kernel
                                launch (plain launches) for pg_last_stats */
   int32_t window_rows;      /* rows of per-round counters kept on the device
@@ -178,7 +182,8 @@ typedef struct {
                                loaded by each lane; 0 or 1 = per-lane loads
                                (the default: they measured faster on a 2^26-
                                node graph with 8-word rows) */
-  int32_t sparse_push;      /* sparse rounds: 0 (default) or 2 = push, each
+  int32_t sparse_push;      /* sparse rounds: 0 (default) or 2 (2: always in
+                               kernels launched round by round) = push, each
                                row that changed in the previous round ORs
                                its delta into its out-neighbours with
                                atomics (their claims for m_active made on

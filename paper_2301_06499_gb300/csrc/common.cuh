@@ -12,6 +12,7 @@
 namespace pg {
 
 constexpr int kBlock = 256;
+constexpr int32_t kStatusWindow = 100;  // device asks the host to move the counts window
 constexpr unsigned kFullMask = 0xFFFFFFFFu;
 
 // Packed frontier append: count of rows in the high bits, running sum of
@@ -52,6 +53,16 @@ struct Ctrl {
   unsigned long long nE_prev;  // out-arc pieces of F_{t-1} (read by a push round)
 };
 
+// Counters and barrier of the resident round loop (resident.cu), on lines of
+// their own; zero when allocated and after a launch that gave up.
+struct ResidentCtl {
+  alignas(128) unsigned long long fp[3];  // F_t by t mod 3: (count << kFsumBits) | out-arc sum
+  alignas(128) unsigned long long ne[3];  // pieces of F_t's long rows
+  alignas(128) uint32_t arrive;           // blocks at the barrier
+  alignas(128) uint32_t gen;              // barriers passed
+  uint32_t abort;                         // a wait ran out
+};
+
 // Per-round work counters (device), indexed by round.
 struct RoundStats {
   unsigned long long work;     // sum over active rows of s_graph(v) * indeg(v)
@@ -86,9 +97,11 @@ struct Params {
   const int32_t *out_col;
   uint64_t *X;  // signatures of round t-1 (read by the pull)
   uint64_t *Y;  // signatures of round t (written by the pull)
+  uint64_t *D2;       // resident loop: D_{t mod 3} (Y is not used)
   uint64_t *D0, *D1;  // deltas: D_{t&1}[v] = bits v gained in round t (0 if unchanged)
   int32_t Wp;   // words per row (padded)
   int32_t s;    // seeds in this pass (valid bits)
+  uint32_t *C2;        // resident loop: C_{t mod 3} (Sat is not used)
   uint32_t *C0, *C1;   // changed-in-round bitmaps, alternating by round parity
   uint32_t *K0, *K1;   // claim / active bitmaps, alternating
   uint32_t *Sat;       // saturated (all s bits set)
@@ -98,6 +111,7 @@ struct Params {
   int32_t pass_words;
   uint32_t *Kw0, *Kw1;  // [Wp][nbm] each (null unless pass_words)
   int64_t nbm;         // 32-bit words per bitmap
+  int32_t *F2;         // resident loop: F_{t mod 3}
   int32_t *F0, *F1;    // rows changed in round t, by round parity
   unsigned long long *E;  // out-arc pieces of F rows: (row << 32) | piece of LE arcs
   unsigned long long *E1; // with push rounds: the pieces of odd rounds (E: even), else null
@@ -134,6 +148,8 @@ struct Params {
   const int32_t *perm;  // relabelled graph: caller id -> internal id (else null)
   int64_t perm_n;       // nodes of the relabelled graph (replicas: a seed k*perm_n + x
                         // of copy k maps to k*perm_n + perm[x])
+  ResidentCtl *rctl;    // resident loop (else null)
+  int32_t row_base;     // resident loop: round in row 0 of the counts window
   RoundStats *rs;       // [row_cap + 2], slot = round - row_base
   Ctrl *ctrl;
   int32_t max_rounds;

@@ -109,6 +109,21 @@ __device__ __forceinline__ void store_words(uint64_t *p, const uint64_t (&a)[CW]
   }
 }
 
+// 32 x 32 bit transpose across a warp: on entry lane r holds row r (bit c =
+// M[r][c]); on exit lane c holds column c (bit r = M[r][c]). Five stages,
+// each swapping the off-diagonal blocks of one bit level.
+__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
+  const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
+#pragma unroll
+  for (int st = 0; st < 5; ++st) {
+    const int j = 16 >> st;
+    const uint32_t m = masks[st];
+    const uint32_t y = __shfl_xor_sync(kFullMask, x, j);
+    x = (lane & j) ? ((x & ~m) | ((y & ~m) >> j)) : ((x & m) | ((y & m) << j));
+  }
+  return x;
+}
+
 // Block-wide sums of N counters, then one atomicAdd per nonzero counter.
 template <int N>
 __device__ __forceinline__ void block_add(const unsigned long long (&v)[N],
@@ -1085,6 +1100,14 @@ __global__ void __launch_bounds__(kBlock, CW <= 4 ? PG_PULL_MIN_BLOCKS : PG_PULL
 }
 
 using PullFn = void (*)(Params);
+// The resident round loop (resident.cu): a cooperative launch of 64 to 1,024
+// threads a block; counters of up to kResidentCounts columns in shared memory.
+constexpr int kResidentCounts = 12288;
+constexpr int kResidentRow = 32;      // out-arcs of a frontier row that one lane pushes
+constexpr int kResidentPiece = 256;   // out-arcs of a longer row per warp
+using ResidentFn = void (*)(Params, const int32_t *, const int32_t *, int, int, int);
+ResidentFn resident_fn(int CW, bool pw);
+size_t resident_smem(int ncols, int threads);
 // Push rounds as a kernel of their own (k_push<CW, PW>, push.cu): 8-word
 // rows, PROPAGATE-S passes as words and packed batches; it returns at once in
 // rounds that are not pushed.

@@ -14,7 +14,6 @@
 
 namespace pg {
 
-constexpr int32_t kStatusWindow = 100;  // device asks the host to move the counts window
 constexpr int kSmemCountMax = 12288;    // per-seed counters kept in shared memory up to this s
 constexpr int kWidePostWords = 16;      // rows of this many words take k_post's tiled part A
 constexpr int kExpandArcs = 8;          // out-arcs per expansion piece (LE)
@@ -143,21 +142,6 @@ __device__ __forceinline__ bool row_full(const uint64_t *row, int Wp, int s) {
     full &= ((__ldg(reinterpret_cast<const unsigned long long *>(row) + w) | ~valid_mask(w, s)) ==
              ~0ULL);
   return full;
-}
-
-// 32 x 32 bit transpose across a warp: on entry lane r holds row r (bit c =
-// M[r][c]); on exit lane c holds column c (bit r = M[r][c]). Five stages,
-// each swapping the off-diagonal blocks of one bit level.
-__device__ __forceinline__ uint32_t transpose32(uint32_t x, int lane) {
-  const uint32_t masks[5] = {0x0000FFFFu, 0x00FF00FFu, 0x0F0F0F0Fu, 0x33333333u, 0x55555555u};
-#pragma unroll
-  for (int st = 0; st < 5; ++st) {
-    const int j = 16 >> st;
-    const uint32_t m = masks[st];
-    const uint32_t y = __shfl_xor_sync(kFullMask, x, j);
-    x = (lane & j) ? ((x & ~m) | ((y & ~m) >> j)) : ((x & m) | ((y & m) << j));
-  }
-  return x;
 }
 
 // ------------------------------------------------------------- k_post
@@ -967,6 +951,86 @@ struct BatchSeg {
   const int64_t *graph_m;     // host, arcs of each graph (per-graph round kinds)
 };
 
+// Blocks and threads of a resident round loop: a block per SM, and about a
+// warp for every 32 rows, so that a small graph's rounds do not wait for warps
+// without work; packed batches share the SMs with the groups that run beside
+// them (four blocks of 256 threads fit).
+static int resident_threads(int64_t n, bool batch) {
+  int64_t t = 128;
+  while (t < (batch ? 256 : 1024) && t * sm_count() < n) t *= 2;
+  return (int)t;
+}
+
+// Raises the dynamic shared memory limit of the resident kernels (once per
+// device, before any launch).
+static void resident_smem_optin() {
+  static std::mutex mu;
+  static uint64_t done = 0;
+  int dev = 0;
+  cudaGetDevice(&dev);
+  std::lock_guard<std::mutex> lk(mu);
+  if (dev < 64 && (done >> dev) & 1ULL) return;
+  for (int cw : {1, 2, 4, 8})
+    for (bool pw : {false, true})
+      cudaFuncSetAttribute((const void *)resident_fn(cw, pw),
+                           cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           (int)resident_smem(kResidentCounts, 1024));
+  if (dev < 64) done |= 1ULL << dev;
+}
+
+// One pass as a cooperative launch of the resident round loop (launched again
+// after each full counts window).
+static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w, bool batch, int sp,
+                              int col0, PassOut &po) {
+  cudaStream_t st = cl.st;
+  pg_status rc;
+  if (!w.rctl.p) {
+    if ((rc = ensure(w.rctl, sizeof(ResidentCtl)))) return rc;
+    if ((rc = cuda_status(cudaMemsetAsync(w.rctl.p, 0, sizeof(ResidentCtl), st)))) return rc;
+  }
+  p.rctl = (ResidentCtl *)w.rctl.p;
+  resident_smem_optin();
+  const ResidentFn fn = resident_fn(pl.CW, pl.pw);
+  const int threads = resident_threads(p.n, batch);
+  const size_t smem = resident_smem(p.ncols, threads);
+  const int32_t *seeds = (const int32_t *)w.seeds.p;
+  const int32_t *bits = batch ? (const int32_t *)w.seed_bits.p : nullptr;
+  int resume = 0;
+  p.row_base = 0;
+  int64_t launches_guard = (int64_t)cl.max_rounds / std::max<int32_t>(p.row_cap, 1) + 4;
+  Ctrl fin{};
+  for (;;) {
+    if (launches_guard-- < 0) return PG_EDEVICE;
+    int epoch = ++w.epoch;
+    void *args[] = {&p, &seeds, &bits, &sp, &resume, &epoch};
+    if ((rc = cuda_status(cudaLaunchCooperativeKernel((const void *)fn, dim3(sm_count()),
+                                                      dim3(threads), args, smem, st))))
+      return rc;
+    po.launches += 1;
+    if ((rc = cuda_status(cudaMemcpyAsync(&w.ctrl_h[0], p.ctrl, sizeof(Ctrl),
+                                          cudaMemcpyDeviceToHost, st))) ||
+        (rc = cuda_status(cudaStreamSynchronize(st))))
+      return rc;
+    fin = w.ctrl_h[0];
+    if (!fin.done || fin.iters != epoch) {  // a wait of the barrier ran out
+      cudaMemsetAsync(w.rctl.p, 0, sizeof(ResidentCtl), st);
+      return PG_ETIMEOUT;
+    }
+    if (fin.status != kStatusWindow) break;
+    if ((rc = copy_window(cl, p, col0, p.row_base, p.row_cap, p.row_cap))) return rc;
+    p.row_base += p.row_cap;
+    resume = 1;
+  }
+  if (fin.bad_index) return PG_EDEVICE;  // a PG_DEBUG_BOUNDS build caught a bad gather
+  const int32_t last = fin.status == PG_ERANGE ? cl.max_rounds : fin.last_round;
+  const int32_t rows = last - p.row_base + 1;
+  if ((rc = copy_window(cl, p, col0, p.row_base, rows, rows + 1))) return rc;
+  po.rounds = fin.status == PG_ERANGE ? cl.max_rounds + 1 : fin.last_round;
+  po.status = fin.status;
+  po.dense_rounds = fin.dense_rounds;
+  return PG_OK;
+}
+
 // One pass: sp seeds of the call, columns [col0, col0+sp); or, with bs, all
 // seeds of a packed batch.
 // With pw, the sp seeds are ceil(sp/64) PROPAGATE-S passes of 64 planes run
@@ -1000,7 +1064,11 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   const int64_t n = g->n;
   const int64_t nbm = (n + 31) / 32;
   const int32_t row_cap = cl.row_cap;
-  const int64_t e_cap = n + g->m / kExpandArcs + 1;
+  // the resident round loop: the default for rows of up to 8 words gathered
+  // whole. The other schedules, and per-launch events, run round by round.
+  const bool resident = !pl.wide && pl.CW == pl.Wp && cl.o.sparse_push == 0 &&
+                        cl.o.use_graphs != 0 && cl.o.timing == 0 && cl.o.tma_gather != 2;
+  const int64_t e_cap = resident ? g->m / kResidentRow + 1 : n + g->m / kExpandArcs + 1;
   const size_t sig_bytes = sizeof(uint64_t) * (size_t)n * pl.Wp;
   const size_t bm_bytes = sizeof(uint32_t) * (size_t)nbm;
   pl.post_wide = !bs && pl.Wp >= kWidePostWords;
@@ -1013,14 +1081,18 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
       {&w.Sat, bm_bytes},
       {&w.F0, sizeof(int32_t) * (size_t)n}, {&w.F1, sizeof(int32_t) * (size_t)n},
       {&w.E, sizeof(unsigned long long) * (size_t)e_cap},
-      {&w.A, sizeof(ulonglong2) * (size_t)std::max<int64_t>(npieces, 1)},
       {&w.counts, sizeof(uint32_t) * (size_t)row_cap * (size_t)ncols},
       {&w.rs, sizeof(RoundStats) * (size_t)(row_cap + 2)},
       {&w.ctrl, sizeof(Ctrl)}, {&w.seeds, sizeof(int32_t) * (size_t)sp}};
+  if (resident)
+    needs.push_back({&w.F2, sizeof(int32_t) * (size_t)n});
+  else
+    needs.push_back({&w.A, sizeof(ulonglong2) * (size_t)std::max<int64_t>(npieces, 1)});
   if (pl.post_wide) needs.push_back({&w.RB, sizeof(uint32_t) * (size_t)n});
-  if (pw) {
-    needs.push_back({&w.KW0, bm_bytes * (size_t)pl.Wp});
-    needs.push_back({&w.KW1, bm_bytes * (size_t)pl.Wp});
+  if (pw) {  // claim bits per (word, row); the resident loop: a byte per row
+    const size_t kw = resident ? ((size_t)n + 3) / 4 * 4 : bm_bytes * (size_t)pl.Wp;
+    needs.push_back({&w.KW0, kw});
+    needs.push_back({&w.KW1, kw});
   }
   if (bs) needs.push_back({&w.seed_bits, sizeof(int32_t) * (size_t)sp});
   // push rounds (rows of up to 8 words gathered whole): the frontier's
@@ -1029,10 +1101,10 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   // 10^6 with s = 128 by 11%, on R-MAT 26 with s = 512 by 10% and on the
   // 512-graph mix (batched) by 3%
   const bool push_ok = !pl.wide && pl.CW == pl.Wp;
-  const bool push = push_ok && cl.o.sparse_push != 1;
+  const bool push = resident || (push_ok && cl.o.sparse_push != 1);
   if (push) needs.push_back({&w.E1, sizeof(unsigned long long) * (size_t)e_cap});
   if (bs && g->nseg > 0) {
-    needs.push_back({&w.gfsum, 2 * sizeof(unsigned long long) * (size_t)g->nseg});
+    needs.push_back({&w.gfsum, 3 * sizeof(unsigned long long) * (size_t)g->nseg});
     needs.push_back({&w.gthr, sizeof(unsigned long long) * (size_t)g->nseg});
     needs.push_back({&w.dlist, sizeof(int32_t) * (size_t)g->nseg});
     needs.push_back({&w.dpref, sizeof(int64_t) * ((size_t)g->nseg + 1)});
@@ -1065,8 +1137,8 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   p.s = s_bits;
   p.C0 = (uint32_t *)w.C0.p;
   p.C1 = (uint32_t *)w.C1.p;
-  p.K0 = (uint32_t *)w.K0.p;
-  p.K1 = (uint32_t *)w.K1.p;
+  p.K0 = (uint32_t *)(resident && pw ? w.KW0.p : w.K0.p);
+  p.K1 = (uint32_t *)(resident && pw ? w.KW1.p : w.K1.p);
   p.Sat = (uint32_t *)w.Sat.p;
   p.rowbits = pl.post_wide ? (uint32_t *)w.RB.p : nullptr;
   p.pass_words = pw ? 1 : 0;
@@ -1130,6 +1202,11 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
                    (cl.o.test_changed == 0 && big);
   p.test_adapt = !p.gfsum && (cl.o.test_changed == 3 || (cl.o.test_changed == 0 && big));
   p.early_stop = g->m >= kEarlyStopArcs;
+  if (resident) {
+    p.D2 = (uint64_t *)w.Y.p;
+    p.C2 = (uint32_t *)w.Sat.p;
+    p.F2 = (int32_t *)w.F2.p;
+  }
   p.use_cond = 0;
   p.cond = 0ULL;
   p.iter_guard = cl.max_rounds + 2;
@@ -1190,7 +1267,8 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
       thr[k] = cl.o.direction == PG_DIR_DENSE    ? 0ULL
                : cl.o.direction == PG_DIR_SPARSE ? ~0ULL
                                                  : (unsigned long long)(f * (double)bs->graph_m[k]);
-    rc = cuda_status(cudaMemsetAsync(p.gfsum, 0, 2 * sizeof(unsigned long long) * g->nseg, st));
+    if (!resident)
+      rc = cuda_status(cudaMemsetAsync(p.gfsum, 0, 2 * sizeof(unsigned long long) * g->nseg, st));
     if (rc == PG_OK)
       rc = cuda_status(cudaMemcpyAsync(w.gthr.p, thr.data(), sizeof(unsigned long long) * g->nseg,
                                        cudaMemcpyHostToDevice, st));
@@ -1200,6 +1278,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
     rc = cuda_status(cudaMemcpyAsync(w.seed_bits.p, bs->seed_bit, sizeof(int32_t) * sp,
                                      cudaMemcpyHostToDevice, st));
   if (rc) return rc;
+  if (resident) return run_resident(cl, pl, p, w, bs != nullptr, sp, col0, po);
   const int64_t count_words = (int64_t)row_cap * ncols;
   const int64_t rs_words = (int64_t)(row_cap + 2) * (int64_t)(sizeof(RoundStats) / 8);
   const int64_t zero_work = std::max<int64_t>({n * pl.Wp / 2, nbm, count_words, rs_words, 1});

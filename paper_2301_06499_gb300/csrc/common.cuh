@@ -58,9 +58,11 @@ struct Ctrl {
 struct ResidentCtl {
   alignas(128) unsigned long long fp[3];  // F_t by t mod 3: (count << kFsumBits) | out-arc sum
   alignas(128) unsigned long long ne[3];  // pieces of F_t's long rows
-  alignas(128) uint32_t arrive;           // blocks at the barrier
-  alignas(128) uint32_t gen;              // barriers passed
-  uint32_t abort;                         // a wait ran out
+  alignas(128) unsigned long long alive[3][8];  // seeds that gained a pair, by t mod 3
+  alignas(128) uint32_t arrive;           // arrivals at the launch's barriers so far
+  alignas(128) uint32_t gen;              // barriers released (packed batches)
+  alignas(128) uint32_t abort;            // a wait ran out
+  uint32_t exited;                        // blocks that left the launch
 };
 
 // Per-round work counters (device), indexed by round.
@@ -101,7 +103,7 @@ struct Params {
   uint64_t *D0, *D1;  // deltas: D_{t&1}[v] = bits v gained in round t (0 if unchanged)
   int32_t Wp;   // words per row (padded)
   int32_t s;    // seeds in this pass (valid bits)
-  uint32_t *C2;        // resident loop: C_{t mod 3} (Sat is not used)
+  uint32_t *C2;        // resident loop: C_{t mod 3} hold two mark bits a row (K, Sat not used)
   uint32_t *C0, *C1;   // changed-in-round bitmaps, alternating by round parity
   uint32_t *K0, *K1;   // claim / active bitmaps, alternating
   uint32_t *Sat;       // saturated (all s bits set)
@@ -149,6 +151,9 @@ struct Params {
   int64_t perm_n;       // nodes of the relabelled graph (replicas: a seed k*perm_n + x
                         // of copy k maps to k*perm_n + perm[x])
   ResidentCtl *rctl;    // resident loop (else null)
+  uint32_t *deg_in, *deg_out;  // resident loop: degrees (the same array for symmetric graphs)
+  int64_t dense_above;  // resident loop: a full sweep when the frontier's out-arcs pass this
+  int32_t col_quads;    // resident loop: out_col is 16-byte aligned
   int32_t row_base;     // resident loop: round in row 0 of the counts window
   RoundStats *rs;       // [row_cap + 2], slot = round - row_base
   Ctrl *ctrl;

@@ -951,13 +951,26 @@ struct BatchSeg {
   const int64_t *graph_m;     // host, arcs of each graph (per-graph round kinds)
 };
 
-// Blocks and threads of a resident round loop: a block per SM, and about a
-// warp for every 32 rows, so that a small graph's rounds do not wait for warps
-// without work; packed batches share the SMs with the groups that run beside
-// them (four blocks of 256 threads fit).
-static int resident_threads(int64_t n, bool batch) {
+// Frontier out-arcs above which a round of the resident loop is a full sweep,
+// as a part of all arcs, where the caller keeps the default. A pushed arc costs
+// several swept ones, but a sweep of a graph without long rows (grids, road
+// networks, uniform random graphs) costs its whole latency: 1024^2 grid
+// (s = 128) 37.1 ms a call at 0.2 against 51.1 at 0.05, ER within 1% either
+// way. With hubs the sends of one long row collide: R-MAT 22 (s = 256) 1.89 ms
+// at 0.05 against 2.14 at 0.2, R-MAT 18 (s = 100) 0.57 against 0.69.
+constexpr int64_t kEvenDegree = 64;
+
+static double resident_threshold(const pg_graph *g, const pg_options &o) {
+  if (o.dense_threshold > 0 && o.dense_threshold != 0.05f) return (double)o.dense_threshold;
+  return g->max_degree <= kEvenDegree ? 0.2 : (double)0.05f;
+}
+
+// Threads per block of a resident round loop of one block per SM: about a warp
+// for every 32 rows, so that a small graph's rounds do not wait for warps
+// without work.
+static int resident_threads(int64_t n, int blocks) {
   int64_t t = 128;
-  while (t < (batch ? 256 : 1024) && t * sm_count() < n) t *= 2;
+  while (t < kResidentThreads && t * blocks < n) t *= 2;
   return (int)t;
 }
 
@@ -971,10 +984,10 @@ static void resident_smem_optin() {
   std::lock_guard<std::mutex> lk(mu);
   if (dev < 64 && (done >> dev) & 1ULL) return;
   for (int cw : {1, 2, 4, 8})
-    for (bool pw : {false, true})
-      cudaFuncSetAttribute((const void *)resident_fn(cw, pw),
+    for (int kind = 0; kind < 3; ++kind)
+      cudaFuncSetAttribute((const void *)resident_fn(cw, kind == 1, kind == 2),
                            cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           (int)resident_smem(kResidentCounts, 1024));
+                           (int)resident_smem(kResidentCounts, kResidentThreads));
   if (dev < 64) done |= 1ULL << dev;
 }
 
@@ -990,8 +1003,11 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   }
   p.rctl = (ResidentCtl *)w.rctl.p;
   resident_smem_optin();
-  const ResidentFn fn = resident_fn(pl.CW, pl.pw);
-  const int threads = resident_threads(p.n, batch);
+  const ResidentFn fn = resident_fn(pl.CW, pl.pw, batch);
+  // the SMs given to this graph (propagations that run side by side share
+  // them: a cooperative launch waits until all its blocks fit), else all
+  const int blocks = cl.g->sms > 0 ? std::min(cl.g->sms, sm_count()) : sm_count();
+  const int threads = resident_threads(p.n, blocks);
   const size_t smem = resident_smem(p.ncols, threads);
   const int32_t *seeds = (const int32_t *)w.seeds.p;
   const int32_t *bits = batch ? (const int32_t *)w.seed_bits.p : nullptr;
@@ -1003,7 +1019,7 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
     if (launches_guard-- < 0) return PG_EDEVICE;
     int epoch = ++w.epoch;
     void *args[] = {&p, &seeds, &bits, &sp, &resume, &epoch};
-    if ((rc = cuda_status(cudaLaunchCooperativeKernel((const void *)fn, dim3(sm_count()),
+    if ((rc = cuda_status(cudaLaunchCooperativeKernel((const void *)fn, dim3(blocks),
                                                       dim3(threads), args, smem, st))))
       return rc;
     po.launches += 1;
@@ -1067,27 +1083,33 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   // the resident round loop: the default for rows of up to 8 words gathered
   // whole. The other schedules, and per-launch events, run round by round.
   const bool resident = !pl.wide && pl.CW == pl.Wp && cl.o.sparse_push == 0 &&
-                        cl.o.use_graphs != 0 && cl.o.timing == 0 && cl.o.tma_gather != 2;
+                        cl.o.use_graphs != 0 && cl.o.timing == 0 && cl.o.tma_gather != 2 &&
+                        (!bs || (g->nseg > 0 && bs->graph_m));
   const int64_t e_cap = resident ? g->m / kResidentRow + 1 : n + g->m / kExpandArcs + 1;
   const size_t sig_bytes = sizeof(uint64_t) * (size_t)n * pl.Wp;
   const size_t bm_bytes = sizeof(uint32_t) * (size_t)nbm;
+  const size_t c_bytes = resident ? 2 * bm_bytes : bm_bytes;  // resident: two mark bits a row
   pl.post_wide = !bs && pl.Wp >= kWidePostWords;
   // the delta buffers keep one all-zero row past the last node (the row a
   // TMA gather of an empty slot reads)
   const size_t delta_bytes_alloc = sig_bytes + sizeof(uint64_t) * (size_t)pl.Wp;
   std::vector<std::pair<DevBuf *, size_t>> needs = {
       {&w.X, sig_bytes}, {&w.Y, sig_bytes}, {&w.D0, delta_bytes_alloc}, {&w.D1, delta_bytes_alloc},
-      {&w.C0, bm_bytes}, {&w.C1, bm_bytes}, {&w.K0, bm_bytes}, {&w.K1, bm_bytes},
-      {&w.Sat, bm_bytes},
+      {&w.C0, c_bytes}, {&w.C1, c_bytes}, {&w.Sat, c_bytes},
       {&w.F0, sizeof(int32_t) * (size_t)n}, {&w.F1, sizeof(int32_t) * (size_t)n},
       {&w.E, sizeof(unsigned long long) * (size_t)e_cap},
       {&w.counts, sizeof(uint32_t) * (size_t)row_cap * (size_t)ncols},
       {&w.rs, sizeof(RoundStats) * (size_t)(row_cap + 2)},
       {&w.ctrl, sizeof(Ctrl)}, {&w.seeds, sizeof(int32_t) * (size_t)sp}};
-  if (resident)
+  if (resident) {
     needs.push_back({&w.F2, sizeof(int32_t) * (size_t)n});
-  else
+    needs.push_back({&w.DI, sizeof(uint32_t) * (size_t)n});
+    if (g->out_ptr != g->row_ptr) needs.push_back({&w.DO, sizeof(uint32_t) * (size_t)n});
+  } else {
+    needs.push_back({&w.K0, bm_bytes});
+    needs.push_back({&w.K1, bm_bytes});
     needs.push_back({&w.A, sizeof(ulonglong2) * (size_t)std::max<int64_t>(npieces, 1)});
+  }
   if (pl.post_wide) needs.push_back({&w.RB, sizeof(uint32_t) * (size_t)n});
   if (pw) {  // claim bits per (word, row); the resident loop: a byte per row
     const size_t kw = resident ? ((size_t)n + 3) / 4 * 4 : bm_bytes * (size_t)pl.Wp;
@@ -1137,8 +1159,8 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   p.s = s_bits;
   p.C0 = (uint32_t *)w.C0.p;
   p.C1 = (uint32_t *)w.C1.p;
-  p.K0 = (uint32_t *)(resident && pw ? w.KW0.p : w.K0.p);
-  p.K1 = (uint32_t *)(resident && pw ? w.KW1.p : w.K1.p);
+  p.K0 = (uint32_t *)w.K0.p;
+  p.K1 = (uint32_t *)w.K1.p;
   p.Sat = (uint32_t *)w.Sat.p;
   p.rowbits = pl.post_wide ? (uint32_t *)w.RB.p : nullptr;
   p.pass_words = pw ? 1 : 0;
@@ -1206,6 +1228,10 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
     p.D2 = (uint64_t *)w.Y.p;
     p.C2 = (uint32_t *)w.Sat.p;
     p.F2 = (int32_t *)w.F2.p;
+    p.deg_in = (uint32_t *)w.DI.p;
+    p.deg_out = g->out_ptr != g->row_ptr ? (uint32_t *)w.DO.p : p.deg_in;
+    p.dense_above = (int64_t)(resident_threshold(g, cl.o) * (double)p.m);
+    p.col_quads = ((uintptr_t)p.out_col & 15) == 0;
   }
   p.use_cond = 0;
   p.cond = 0ULL;

@@ -48,6 +48,7 @@ namespace {
 
 constexpr int kBigRow = kResidentRow;
 constexpr int kBigPiece = kResidentPiece;
+constexpr int kMaxThreads = kResidentThreads;
 constexpr int kStage = 256;      // staged frontier rows per warp
 constexpr unsigned long long kBarrierNs = 20ULL * 1000 * 1000 * 1000;
 
@@ -84,8 +85,18 @@ __device__ __forceinline__ void ld_row(uint64_t (&a)[CW], const uint64_t *p) {
 __device__ __forceinline__ uint32_t ld_u32(const uint32_t *p) {
   return *((volatile const uint32_t *)p);
 }
-__device__ __forceinline__ bool bit_live(const uint32_t *bm, int64_t v) {
-  return (ld_u32(bm + (v >> 5)) >> (v & 31)) & 1u;
+// Row marks of a round, two bits a row: claimed (counted in m_active) and
+// changed (in F_t). One atomic sets and tells both.
+constexpr uint32_t kClaimed = 1u, kChanged = 2u;
+// (mark_word: the row's whole word, so that several can be under way.)
+__device__ __forceinline__ uint32_t mark_word(uint32_t *M, int64_t v, uint32_t bits) {
+  return atomicOr(M + (v >> 4), bits << ((v & 15) * 2));
+}
+__device__ __forceinline__ uint32_t mark(uint32_t *M, int64_t v, uint32_t bits) {
+  return mark_word(M, v, bits) >> ((v & 15) * 2);
+}
+__device__ __forceinline__ bool changed(const uint32_t *M, int64_t v) {
+  return ((M[v >> 4] >> ((v & 15) * 2)) & kChanged) != 0u;
 }
 
 __device__ __forceinline__ uint32_t ld_acquire(const uint32_t *p) {
@@ -107,15 +118,15 @@ __device__ __forceinline__ void red_or(uint64_t *p, uint64_t v) {
 
 // Per-block state: the staged rows' totals of each warp, the round's counters.
 struct Shared {
-  unsigned long long od[32], ne[32];
-  int cnt[32];
+  unsigned long long od, ne;  // out-arcs and pieces of the block's staged rows
   unsigned long long base_f, base_e;
   unsigned long long mact, work;
-  uint32_t rows;
+  uint32_t rows, staged;
   uint64_t alive[kAliveWords];
-  int last;    // this block arrived last
-  int failed;  // the barrier gave up
   unsigned long long fp, ne_all;
+  uint32_t bar;  // barriers this block has arrived at
+  int last;      // this block arrived last
+  int failed;    // the barrier gave up
 };
 
 // Per-thread state of one round.
@@ -126,14 +137,19 @@ struct Lane {
   int t, cur;            // round, its delta buffer
   const uint64_t *Dp;    // deltas of round t-1
   uint64_t *Dc;          // deltas of round t
-  const uint32_t *Cp;
-  uint32_t *Cc, *Kc;
+  const uint32_t *Mp;    // marks of round t-1
+  uint32_t *Mc;          // marks of round t
+  uint32_t *Kc;          // passes as words: claim bytes of round t
   int32_t *F;            // F_t
   unsigned long long *E; // pieces of F_t's long rows
-  uint32_t *cnt;         // counters of this round: shared memory, or the counts row
+  uint32_t cs;           // counters of this round: shared-memory address,
+  uint32_t *cg;          // or (cs = 0) the counts row
   int32_t *stage;
   int scnt;
   bool pieces;           // append E_t (a round that may be followed by a push)
+  unsigned long long od, ne;  // out-arcs and pieces of the rows staged by this lane
+  int gcur;                   // a packed batch: graph and out-arcs not yet added to its sum
+  unsigned long long gacc;
   unsigned long long mact, work;
   uint32_t rows;
   // over the whole launch
@@ -143,103 +159,117 @@ struct Lane {
 __device__ __forceinline__ uint64_t *delta_buf(const Params &p, int k) {
   return k == 0 ? p.D0 : k == 1 ? p.D1 : p.D2;
 }
-__device__ __forceinline__ uint32_t *changed_buf(const Params &p, int k) {
+__device__ __forceinline__ uint32_t *mark_buf(const Params &p, int k) {
   return k == 0 ? p.C0 : k == 1 ? p.C1 : p.C2;
 }
 __device__ __forceinline__ int32_t *frontier_buf(const Params &p, int k) {
   return k == 0 ? p.F0 : k == 1 ? p.F1 : p.F2;
 }
 
-// Grid barrier. With a finalizer (a packed batch) the block that arrives last
-// runs it before the others go on. Returns false once any block gave up.
-template <class Fin>
+// Waits until *word, counting up, reaches target (modulo 2^32).
+__device__ __forceinline__ bool wait_for(ResidentCtl *rc, const uint32_t *word, uint32_t target) {
+  unsigned long long t0 = 0;
+  for (int spin = 0; (int32_t)(ld_acquire(word) - target) < 0; ++spin) {
+    if ((spin & 255) == 255) {
+      const unsigned long long t = now_ns();
+      if (!t0) t0 = t;
+      if (ld_acquire(&rc->abort) || t - t0 > kBarrierNs) {
+        st_release(&rc->abort, 1u);  // the host reads it: the call never reports done
+        return false;
+      }
+    }
+  }
+  return true;
+}
+
+// Grid barrier number sh.bar of the launch. Blocks count up one word and wait
+// for it to reach the next multiple of the grid: no answer to wait for before
+// the word can be polled, no release by a last block (about 1.2 us less a
+// round than an arrival counter with a generation word). With a finalizer (a
+// packed batch) the block that arrives last runs it and then releases the
+// others. Returns false once any block gave up.
+template <bool SEG, class Fin>
 __device__ __forceinline__ bool grid_barrier(const Params &p, Shared &sh, Fin fin) {
   ResidentCtl *rc = p.rctl;
   __syncthreads();
-  uint32_t gen = 0;
-  if (threadIdx.x == 0) {
-    gen = ld_acquire(&rc->gen);
-    __threadfence();
-    sh.last = atomicAdd(&rc->arrive, 1u) == gridDim.x - 1;
-    sh.failed = 0;
-  }
-  if (p.gfsum) {  // the last block lists the graphs to sweep
+  if constexpr (SEG) {
+    if (threadIdx.x == 0) {
+      ++sh.bar;
+      __threadfence();
+      sh.last = atomicAdd(&rc->arrive, 1u) + 1u == sh.bar * gridDim.x;
+    }
     __syncthreads();
     if (sh.last) {
       __threadfence();
       fin();
       __syncthreads();
     }
-  }
-  if (threadIdx.x == 0) {
-    if (sh.last) {
-      rc->arrive = 0u;
-      __threadfence();
-      st_release(&rc->gen, gen + 1u);
-    } else {
-      unsigned long long t0 = 0;
-      for (int spin = 0; ld_acquire(&rc->gen) == gen; ++spin) {
-        if ((spin & 255) == 255) {
-          const unsigned long long t = now_ns();
-          if (!t0) t0 = t;
-          if (ld_acquire(&rc->abort) || t - t0 > kBarrierNs) {
-            st_release(&rc->abort, 1u);  // the host reads it: the call never reports done
-            sh.failed = 1;
-            break;
-          }
-        }
+    if (threadIdx.x == 0) {
+      sh.failed = 0;
+      if (sh.last) {
+        __threadfence();
+        st_release(&rc->gen, sh.bar);
+      } else {
+        sh.failed = !wait_for(rc, &rc->gen, sh.bar);
       }
+      __threadfence();
     }
+  } else if (threadIdx.x == 0) {
+    ++sh.bar;
+    __threadfence();
+    atomicAdd(&rc->arrive, 1u);
+    sh.failed = !wait_for(rc, &rc->arrive, sh.bar * gridDim.x);
     __threadfence();
   }
   __syncthreads();
   return !sh.failed;
 }
 
-// Out-degree and piece totals of the warp's staged rows (and, in a packed
-// batch, their graphs' frontier sums).
-__device__ __forceinline__ void stage_totals(const Params &p, const Lane &L, unsigned long long &od_t,
+// A row staged by this lane: its out-arcs (od), for the choice of the next
+// round, and its pieces; in a packed batch, for its graph g's own choice.
+template <bool SEG>
+__device__ __forceinline__ void stage_degree(const Params &p, Lane &L, uint32_t od, int g) {
+  L.od += od;
+  if (od > kBigRow) L.ne += (od + kBigPiece - 1) / kBigPiece;
+  if (SEG && od) {
+    if (g != L.gcur) {
+      if (L.gacc) atomicAdd(p.gfsum + (size_t)L.cur * (size_t)p.nseg + L.gcur, L.gacc);
+      L.gcur = g;
+      L.gacc = 0;
+    }
+    L.gacc += od;
+  }
+}
+
+// Out-arcs and pieces of the warp's staged rows (and, in a packed batch,
+// their graphs' frontier sums).
+template <bool SEG>
+__device__ __forceinline__ void stage_totals(const Params &p, Lane &L, unsigned long long &od_t,
                                              unsigned long long &ne_t) {
   __syncwarp();
-  unsigned long long od_l = 0, ne_l = 0, gacc = 0;
-  unsigned long long *gf = p.gfsum ? p.gfsum + (size_t)L.cur * (size_t)p.nseg : nullptr;
-  int gcur = -1;
-  for (int i = L.lane; i < L.scnt; i += 32) {
-    const int32_t v = L.stage[i];
-    const unsigned long long od =
-        (unsigned long long)(__ldg(p.out_ptr + v + 1) - __ldg(p.out_ptr + v));
-    od_l += od;
-    if (od > kBigRow) ne_l += (od + kBigPiece - 1) / kBigPiece;
-    if (gf && od) {
-      const int gq = __ldg(p.node_graph + v);
-      if (gq != gcur) {
-        if (gacc) atomicAdd(gf + gcur, gacc);
-        gcur = gq;
-        gacc = 0;
-      }
-      gacc += od;
-    }
-  }
-  if (gf) {  // one atomic per warp when its lanes ended on one graph
-    const unsigned has = __ballot_sync(kFullMask, gacc != 0);
+  if constexpr (SEG) {  // one atomic per warp when its lanes ended on one graph
+    unsigned long long *gf = p.gfsum + (size_t)L.cur * (size_t)p.nseg;
+    const unsigned has = __ballot_sync(kFullMask, L.gacc != 0);
     if (has) {
-      const int g0 = __shfl_sync(kFullMask, gcur, __ffs(has) - 1);
-      if (__all_sync(kFullMask, gacc == 0 || gcur == g0)) {
+      const int g0 = __shfl_sync(kFullMask, L.gcur, __ffs(has) - 1);
+      if (__all_sync(kFullMask, L.gacc == 0 || L.gcur == g0)) {
         unsigned long long tot;
-        warp_excl_scan64(gacc, L.lane, &tot);
+        warp_excl_scan64(L.gacc, L.lane, &tot);
         if (L.lane == 0) atomicAdd(gf + g0, tot);
-      } else if (gacc) {
-        atomicAdd(gf + gcur, gacc);
+      } else if (L.gacc) {
+        atomicAdd(gf + L.gcur, L.gacc);
       }
     }
+    L.gacc = 0;
   }
+  od_t = L.od;
+  ne_t = L.pieces ? L.ne : 0ULL;
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
-    od_l += __shfl_xor_sync(kFullMask, od_l, off);
-    ne_l += __shfl_xor_sync(kFullMask, ne_l, off);
+    od_t += __shfl_xor_sync(kFullMask, od_t, off);
+    ne_t += __shfl_xor_sync(kFullMask, ne_t, off);
   }
-  od_t = od_l;
-  ne_t = L.pieces ? ne_l : 0ULL;
+  L.od = L.ne = 0;
 }
 
 // Writes the warp's staged rows at F[bf] and their pieces at E[be].
@@ -265,9 +295,10 @@ __device__ __forceinline__ void stage_write(const Params &p, const Lane &L, unsi
 }
 
 // A full stage in the middle of a round: the warp reserves its own places.
+template <bool SEG>
 __device__ __forceinline__ void stage_spill(const Params &p, Lane &L) {
   unsigned long long od_t, ne_t, bf = 0, be = 0;
-  stage_totals(p, L, od_t, ne_t);
+  stage_totals<SEG>(p, L, od_t, ne_t);
   if (L.lane == 0) {
     bf = atomicAdd(&p.rctl->fp[L.cur], ((unsigned long long)L.scnt << kFsumBits) + od_t);
     if (ne_t) be = atomicAdd(&p.rctl->ne[L.cur], ne_t);
@@ -288,83 +319,81 @@ __device__ __forceinline__ void stage_row(Lane &L, int32_t v, bool app) {
 // The end of a round's work: the block's staged rows with one reservation for
 // all its warps (a warp each would queue at the counters: same-address
 // atomics take about 0.65 ns each), its counts and work sums.
+template <bool PW, bool SEG>
 __device__ __forceinline__ void round_flush(const Params &p, Lane &L, Shared &sh, uint32_t *scnt_s) {
-  unsigned long long od_t, ne_t;
-  stage_totals(p, L, od_t, ne_t);
-  unsigned long long m = L.mact, w = L.work, r = L.rows;
+  unsigned long long od_t = 0, ne_t = 0;
+  if (L.scnt) stage_totals<SEG>(p, L, od_t, ne_t);
+  if (__any_sync(kFullMask, L.rows != 0u)) {
+    unsigned long long m = L.mact, w = L.work;
+    uint32_t r = __reduce_add_sync(kFullMask, L.rows);
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) {
-    m += __shfl_xor_sync(kFullMask, m, off);
-    w += __shfl_xor_sync(kFullMask, w, off);
-    r += __shfl_xor_sync(kFullMask, r, off);
-  }
-  if (L.lane == 0) {
-    sh.cnt[L.wid] = L.scnt;
-    sh.od[L.wid] = od_t;
-    sh.ne[L.wid] = ne_t;
-    if (r) {
+    for (int off = 16; off > 0; off >>= 1) m += __shfl_xor_sync(kFullMask, m, off);
+    if (PW || SEG) {
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) w += __shfl_xor_sync(kFullMask, w, off);
+    } else {
+      w = m * (unsigned long long)p.s;
+    }
+    if (L.lane == 0) {
       atomicAdd(&sh.mact, m);
       atomicAdd(&sh.work, w);
-      atomicAdd(&sh.rows, (uint32_t)r);
+      atomicAdd(&sh.rows, r);
     }
   }
+  uint32_t at = 0;
+  unsigned long long ae = 0;
+  if (L.lane == 0 && L.scnt) {  // the warp's place among the block's rows
+    at = atomicAdd(&sh.staged, (uint32_t)L.scnt);
+    atomicAdd(&sh.od, od_t);
+    if (ne_t) ae = atomicAdd(&sh.ne, ne_t);
+  }
+  at = __shfl_sync(kFullMask, at, 0);
+  ae = __shfl_sync(kFullMask, ae, 0);
   __syncthreads();
-  const int nw = blockDim.x >> 5;
   RoundStats *rs = p.rs + (L.t - p.row_base);
-  if (L.wid == 0) {  // one reservation for the block
-    const unsigned long long c = L.lane < nw ? (unsigned long long)sh.cnt[L.lane] : 0ULL;
-    const unsigned long long o = L.lane < nw ? sh.od[L.lane] : 0ULL;
-    const unsigned long long e = L.lane < nw ? sh.ne[L.lane] : 0ULL;
-    unsigned long long ct, ot, et;
-    const unsigned long long cx = warp_excl_scan64(c, L.lane, &ct);
-    warp_excl_scan64(o, L.lane, &ot);
-    const unsigned long long ex = warp_excl_scan64(e, L.lane, &et);
+  if (threadIdx.x == 0) {  // one reservation for the block
     unsigned long long bf = 0, be = 0;
-    if (L.lane == 0) {
-      if (et) be = atomicAdd(&p.rctl->ne[L.cur], et);
-      if (ct) bf = atomicAdd(&p.rctl->fp[L.cur], (ct << kFsumBits) + ot) >> kFsumBits;
-    }
-    bf = __shfl_sync(kFullMask, bf, 0);
-    be = __shfl_sync(kFullMask, be, 0);
-    if (L.lane < nw) {
-      sh.od[L.lane] = bf + cx;
-      sh.ne[L.lane] = be + ex;
-    }
-  } else if (L.wid == 1 || nw == 1) {
-    if (L.lane == 0 && sh.rows) {
+    if (sh.staged) bf = atomicAdd(&p.rctl->fp[L.cur], ((unsigned long long)sh.staged << kFsumBits) + sh.od);
+    if (sh.ne) be = atomicAdd(&p.rctl->ne[L.cur], sh.ne);
+    if (sh.rows) {
       atomicAdd(&rs->m_active, sh.mact);
       atomicAdd(&rs->work, sh.work);
       atomicAdd(&rs->rows, (unsigned long long)sh.rows);
     }
+    sh.base_f = bf >> kFsumBits;
+    sh.base_e = be;
+    sh.mact = sh.work = sh.od = sh.ne = 0;
+    sh.rows = sh.staged = 0;
   }
-  if (scnt_s) {
-    uint32_t *crow = p.counts + (size_t)(L.t - p.row_base) * (size_t)p.ncols;
-    for (int i = threadIdx.x; i < p.ncols; i += blockDim.x) {
-      const uint32_t c = scnt_s[i];
-      if (c) {
-        atomicAdd(&crow[i], c);
-        scnt_s[i] = 0u;
-      }
+  if (!SEG && p.early_stop) {  // the seeds that gained a pair
+    for (int w = L.wid; w * 64 < p.ncols; w += blockDim.x >> 5) {
+      const int i = w * 64 + L.lane;
+      const unsigned lo = __ballot_sync(kFullMask, i < p.ncols && scnt_s[i] != 0u);
+      const unsigned hi = __ballot_sync(kFullMask, i + 32 < p.ncols && scnt_s[i + 32] != 0u);
+      if (L.lane == 0 && (lo | hi)) atomicOr(&p.rctl->alive[L.cur][w], ((unsigned long long)hi << 32) | lo);
     }
   }
   __syncthreads();
-  if (L.scnt) stage_write(p, L, sh.od[L.wid], sh.ne[L.wid], ne_t);
+  if (L.scnt) stage_write(p, L, sh.base_f + at, sh.base_e + ae, ne_t);
   L.scnt = 0;
   L.mact = L.work = 0;
   L.rows = 0;
-  if (threadIdx.x == 0) {
-    sh.mact = sh.work = 0;
-    sh.rows = 0;
-  }
+}
+
+__device__ __forceinline__ void count_add(const Lane &L, int col, uint32_t x) {
+  if (L.cs)
+    asm volatile("red.shared.add.u32 [%0], %1;" : : "r"(L.cs + 4u * (uint32_t)col), "r"(x) : "memory");
+  else
+    atomicAdd(L.cg + col, x);
 }
 
 // Counts the bits of each lane's nw (word k of a row whose count columns
 // start at c0): one bit per finder, a handful per row in a sparse round.
-__device__ __forceinline__ void count_bits(uint32_t *cnt, int c0, int k, uint64_t nw) {
+__device__ __forceinline__ void count_bits(const Lane &L, int c0, int k, uint64_t nw) {
   while (nw) {
     const int b = __ffsll((long long)nw) - 1;
     nw &= nw - 1;
-    atomicAdd(cnt + c0 + k * 64 + b, 1u);
+    count_add(L, c0 + k * 64 + b, 1u);
   }
 }
 
@@ -381,136 +410,191 @@ __device__ __forceinline__ uint32_t claim_passes(uint32_t *Kb, int64_t v, uint32
 }
 
 // ------------------------------------------------------------ sparse rounds
-template <int CW, bool PW>
+// A lane holds at most two words of a row: rows of 4 and 8 words take 2 and 4
+// lanes, so that four out-arcs a lane fit the registers at every width. The
+// loads of the four arcs are issued together, then their atomics, then the
+// atomics and loads that depend on those: a frontier row of four arcs costs
+// five dependent accesses, not five per arc.
+template <int CW, bool PW, bool SEG>
 __device__ __forceinline__ void push_round(const Params &p, Lane &L, const int32_t *Fp,
                                            const unsigned long long *Ep, int64_t nF, int64_t nE) {
-  // arcs a lane handles together; the signatures of 8-word rows fill the
-  // registers two at a time
-  constexpr int UNR = CW <= 2 ? 4 : (CW == 4 ? 2 : 1);
-  const size_t Wp = CW;
-  const int64_t groups = (nF + 31) >> 5;
+  constexpr int UNR = 4;                  // out-arcs a lane handles together
+  constexpr int WL = CW <= 2 ? CW : 2;    // words of a row per lane
+  constexpr int SUB = CW / WL;            // lanes per row
+  constexpr int ROWS = 32 / SUB;          // rows per warp
+  const int sub = L.lane % SUB, r = L.lane / SUB, w0 = sub * WL;
+  // a small frontier spreads each row's arcs over more lanes, so that its
+  // rows of up to kBigRow arcs take one step
+  int gl = 0;  // log2 of the lane groups per row
+  while (gl < 3 && (nF * SUB << (gl + 1)) <= L.nth) ++gl;
+  const int rows = ROWS >> gl;  // rows per warp
+  const int64_t groups = (nF + rows - 1) / rows;
   const unsigned long long *gfp =
-      p.gfsum ? p.gfsum + (size_t)((L.t + 2) % 3) * (size_t)p.nseg : nullptr;
+      SEG ? p.gfsum + (size_t)((L.t + 2) % 3) * (size_t)p.nseg : nullptr;
   for (int64_t it = L.warp; it < groups + nE; it += L.nwarps) {
     int32_t u = -1;
     int64_t ob = 0, oe = 0;
     int stride = 1;
     if (it < groups) {
-      const int64_t i = it * 32 + L.lane;
+      const int64_t i = it * rows + (r >> gl);
+      stride = 1 << gl;
       if (i < nF) {
         u = Fp[i];
         ob = __ldg(p.out_ptr + u);
         oe = __ldg(p.out_ptr + u + 1);
         if (oe - ob > kBigRow) oe = ob;  // in pieces, below
+        ob += r & (stride - 1);
       }
     } else {
       const unsigned long long e = Ep[it - groups];
       u = (int32_t)(e >> 32);
       const int64_t b0 = __ldg(p.out_ptr + u) + (int64_t)(e & 0xFFFFFFFFULL) * kBigPiece;
       oe = min(__ldg(p.out_ptr + u + 1), b0 + kBigPiece);
-      ob = b0 + L.lane;
-      stride = 32;
+      ob = b0 + r;
+      stride = ROWS;
     }
-    int gs = p.s, c0 = 0;
+    int gs = p.s, c0 = 0, g = 0;
     unsigned long long *gm = nullptr;
-    if (p.node_graph && u >= 0) {
-      const int g = __ldg(p.node_graph + u);
+    if (SEG && u >= 0) {
+      g = __ldg(p.node_graph + u);
       // a packed batch: graphs swept whole in this round take no push
-      if (gfp && gfp[g] > __ldg(p.gthr + g)) oe = ob;
+      if (gfp[g] > __ldg(p.gthr + g)) oe = ob;
       gs = __ldg(p.graph_s + g);
       c0 = __ldg(p.graph_col0 + g);
       if (p.gmact) gm = p.gmact + (size_t)(L.t - p.row_base) * (size_t)p.nseg + g;
     }
-    uint64_t d[CW];
+    uint64_t d[WL];
 #pragma unroll
-    for (int k = 0; k < CW; ++k) d[k] = 0ULL;
-    if (ob < oe) {
-      if (gather_ok(p, u, CW - 1)) ld_row<CW>(d, L.Dp + (size_t)u * Wp);
-      ++L.items;
-      ++L.gath;
+    for (int k = 0; k < WL; ++k) d[k] = 0ULL;
+    if (ob < oe && gather_ok(p, u, CW - 1)) {
+      ld_row<WL>(d, L.Dp + (size_t)u * CW + w0);
+      if (sub == 0) {
+        ++L.items;
+        ++L.gath;
+      }
     }
     while (__any_sync(kFullMask, ob < oe)) {
       int32_t v[UNR];
-      uint64_t x[UNR][CW];
-      uint32_t kw[UNR];
+      uint64_t x[UNR][WL];
+      uint32_t deg[UNR], bits = 0;
+      if (stride == 1 && p.col_quads && (ob & ~3LL) + 8 <= p.m) {
+        // a row's next four arcs: the two 16-byte quads that hold them
+        int4 lo = make_int4(-1, -1, -1, -1), hi = lo;
+        if (ob < oe) {
+          const int4 *c4 = reinterpret_cast<const int4 *>(p.out_col) + (ob >> 2);
+          lo = __ldg(c4);
+          if (((ob & 3) + (oe - ob)) > 4) hi = __ldg(c4 + 1);
+        }
+        if (ob & 1) lo.x = lo.y, lo.y = lo.z, lo.z = lo.w, lo.w = hi.x, hi.x = hi.y, hi.y = hi.z;
+        if (ob & 2) lo.x = lo.z, lo.y = lo.w, lo.z = hi.x, lo.w = hi.y;
+        v[0] = lo.x, v[1] = lo.y, v[2] = lo.z, v[3] = lo.w;
+#pragma unroll
+        for (int q = 0; q < UNR; ++q)
+          if (ob + q >= oe) v[q] = -1;
+      } else {
+#pragma unroll
+        for (int q = 0; q < UNR; ++q) {
+          const int64_t j = ob + (int64_t)q * stride;
+          v[q] = j < oe ? __ldg(p.out_col + j) : -1;
+        }
+      }
 #pragma unroll
       for (int q = 0; q < UNR; ++q) {
-        const int64_t j = ob + (int64_t)q * stride;
-        v[q] = j < oe ? __ldg(p.out_col + j) : -1;
         if (v[q] >= 0 && !gather_ok(p, v[q], CW - 1)) v[q] = -1;
-      }
+        deg[q] = 0;
 #pragma unroll
-      for (int q = 0; q < UNR; ++q) {
-        kw[q] = 0;
-#pragma unroll
-        for (int k = 0; k < CW; ++k) x[q][k] = ~0ULL;
+        for (int k = 0; k < WL; ++k) x[q][k] = ~0ULL;
         if (v[q] >= 0) {
-          ++L.scan;
-          ld_row<CW>(x[q], p.X + (size_t)v[q] * Wp);
-          if (!PW) kw[q] = ld_u32(L.Kc + (v[q] >> 5));
-        }
-      }
-      // claims (m_active): rows with a zero bit left
-#pragma unroll
-      for (int q = 0; q < UNR; ++q) {
-        if (v[q] < 0) continue;
-        if constexpr (PW) {
-          uint32_t mask = 0;
-#pragma unroll
-          for (int k = 0; k < CW; ++k)
-            if (d[k] && (x[q][k] | ~valid_mask(k, p.s)) != ~0ULL) mask |= 1u << k;
-          if (mask) mask = claim_passes(L.Kc, v[q], mask);
-          if (mask) {
-            const unsigned long long deg =
-                (unsigned long long)(__ldg(p.row_ptr + v[q] + 1) - __ldg(p.row_ptr + v[q]));
-            L.mact += deg * __popc(mask);
-            L.rows += __popc(mask);
-            for (; mask; mask &= mask - 1)
-              L.work += deg * __popcll(valid_mask(__ffs(mask) - 1, p.s));
-          }
-        } else {
-          bool full = true;
-#pragma unroll
-          for (int k = 0; k < CW; ++k) full &= (x[q][k] | ~valid_mask(k, gs)) == ~0ULL;
-          if (full) {
-            v[q] = -1;
-          } else if (!((kw[q] >> (v[q] & 31)) & 1u) && !set_bit(L.Kc, v[q])) {
-            const unsigned long long deg =
-                (unsigned long long)(__ldg(p.row_ptr + v[q] + 1) - __ldg(p.row_ptr + v[q]));
-            L.mact += deg;
-            L.work += deg * (unsigned long long)gs;
-            ++L.rows;
-            if (gm) atomicAdd(gm, deg);
+          ld_row<WL>(x[q], p.X + (size_t)v[q] * CW + w0);
+          if (sub == 0) {
+            ++L.scan;
+            deg[q] = p.deg_in[v[q]];
           }
         }
       }
-      // the bits each row lacks
+      // rows with a zero bit left (PW: per pass, and only passes sent to),
+      // over the row's lanes
 #pragma unroll
-      for (int q = 0; q < UNR; ++q) {
+      for (int q = 0; q < UNR; ++q)
 #pragma unroll
-        for (int k = 0; k < CW; ++k) {
-          const uint64_t g = v[q] >= 0 ? d[k] & ~x[q][k] : 0ULL;
-          x[q][k] = 0ULL;
-          if (g)
-            x[q][k] = g & ~(uint64_t)atomicOr(
-                               reinterpret_cast<unsigned long long *>(p.X + (size_t)v[q] * Wp + k),
-                               (unsigned long long)g);
+        for (int k = 0; k < WL; ++k) {
+          const bool room = (x[q][k] | ~valid_mask(w0 + k, gs)) != ~0ULL;
+          if constexpr (PW) {
+            if (room && d[k]) bits |= 1u << (8 * q + w0 + k);
+          } else {
+            if (room) bits |= 1u << q;
+          }
         }
-      }
 #pragma unroll
-      for (int q = 0; q < UNR; ++q) {
-        bool app = false;
+      for (int off = SUB >> 1; off > 0; off >>= 1) bits |= __shfl_xor_sync(kFullMask, bits, off);
+      // the bits each row lacks: all atomics under way at once
+      uint64_t old[UNR][WL];
 #pragma unroll
-        for (int k = 0; k < CW; ++k)
+      for (int q = 0; q < UNR; ++q)
+#pragma unroll
+        for (int k = 0; k < WL; ++k) {
+          x[q][k] = v[q] >= 0 ? d[k] & ~x[q][k] : 0ULL;
+          old[q][k] = 0ULL;
+          if (x[q][k])
+            old[q][k] = (uint64_t)atomicOr(
+                reinterpret_cast<unsigned long long *>(p.X + (size_t)v[q] * CW + w0 + k),
+                (unsigned long long)x[q][k]);
+        }
+      // new bits: each has this lane as its only finder
+      uint32_t gain = 0;
+#pragma unroll
+      for (int q = 0; q < UNR; ++q)
+#pragma unroll
+        for (int k = 0; k < WL; ++k) {
+          x[q][k] &= ~old[q][k];
           if (x[q][k]) {
-            red_or(L.Dc + (size_t)v[q] * Wp + k, x[q][k]);
-            app = true;
+            red_or(L.Dc + (size_t)v[q] * CW + w0 + k, x[q][k]);
+            gain |= 1u << q;
           }
-        if (app) app = !bit_live(L.Cc, v[q]) && !set_bit(L.Cc, v[q]);
-        if (L.scnt > kStage - 32) stage_spill(p, L);
-        stage_row(L, v[q], app);
+        }
 #pragma unroll
-        for (int k = 0; k < CW; ++k) count_bits(L.cnt, c0, k, x[q][k]);
+      for (int off = SUB >> 1; off > 0; off >>= 1) gain |= __shfl_xor_sync(kFullMask, gain, off);
+      // the claim and the place in F_t, for rows with room
+      uint32_t mk[UNR], od[UNR];
+#pragma unroll
+      for (int q = 0; q < UNR; ++q) {
+        mk[q] = ~0u;
+        od[q] = deg[q];
+        const bool gq = (gain >> q) & 1u;
+        if (sub == 0 && (PW ? gq : ((bits >> q) & 1u) != 0u)) {
+          mk[q] = mark_word(L.Mc, v[q], gq ? kClaimed | kChanged : kClaimed);
+          if (gq && p.deg_out != p.deg_in) od[q] = p.deg_out[v[q]];
+        }
+      }
+#pragma unroll
+      for (int q = 0; q < UNR; ++q)
+#pragma unroll
+        for (int k = 0; k < WL; ++k) count_bits(L, c0, w0 + k, x[q][k]);
+#pragma unroll
+      for (int q = 0; q < UNR; ++q) {
+        mk[q] >>= (v[q] & 15) * 2;
+        if constexpr (PW) {
+          uint32_t m = (bits >> (8 * q)) & 0xFFu;
+          if (sub == 0 && m) m = claim_passes(L.Kc, v[q], m);
+          if (sub == 0 && m) {
+            L.mact += (unsigned long long)deg[q] * __popc(m);
+            L.rows += __popc(m);
+            for (; m; m &= m - 1)
+              L.work += (unsigned long long)deg[q] * __popcll(valid_mask(__ffs(m) - 1, p.s));
+          }
+        } else if (!(mk[q] & kClaimed)) {
+          L.mact += deg[q];
+          if (SEG) L.work += (unsigned long long)deg[q] * (unsigned long long)gs;
+          ++L.rows;
+          if (SEG && gm) atomicAdd(gm, (unsigned long long)deg[q]);
+        }
+      }
+      if (L.scnt > kStage - UNR * ROWS) stage_spill<SEG>(p, L);
+#pragma unroll
+      for (int q = 0; q < UNR; ++q) {
+        const bool app = ((gain >> q) & 1u) && !(mk[q] & kChanged);  // mk is set on sub 0
+        if (app) stage_degree<SEG>(p, L, od[q], g);
+        stage_row(L, v[q], app);
       }
       ob += (int64_t)UNR * stride;
     }
@@ -521,25 +605,25 @@ __device__ __forceinline__ void push_round(const Params &p, Lane &L, const int32
 // The sweep of pull_dense (kernels.cuh) with its early stop, finishing each
 // row on the spot: new bits go to X and D of this round and are counted by a
 // 32 x 32 bit transpose per word and half.
-template <int CW, bool PW>
+template <int CW, bool PW, bool SEG>
 __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
                                             const uint64_t *alive) {
-  constexpr int U = 4;
+  constexpr int U = CW <= 4 && !SEG ? 8 : 4;
   constexpr bool kPipe = CW <= 4;  // at 8 words the registers are not there
   const size_t Wp = CW;
-  const int nd = p.dlist ? *(volatile int32_t *)&p.ctrl->ndense : 0;
-  const int64_t nchunks = p.dlist ? *(volatile int64_t *)(p.dpref + nd) : p.sell_chunks;
+  const int nd = SEG ? *(volatile int32_t *)&p.ctrl->ndense : 0;
+  const int64_t nchunks = SEG ? *(volatile int64_t *)(p.dpref + nd) : p.sell_chunks;
   for (int64_t ci = L.warp; ci < nchunks; ci += L.nwarps) {
     int64_t c = ci;
-    int gs = p.s, c0 = 0;
+    int gs = p.s, c0 = 0, g = 0;
     unsigned long long *gm = nullptr;
-    if (p.dlist) {  // the chunks of the graphs in a full sweep
+    if constexpr (SEG) {  // the chunks of the graphs in a full sweep
       int lo = 0, hi = nd - 1;  // the last k with dpref[k] <= ci
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (*(volatile int64_t *)(p.dpref + mid) <= ci) lo = mid; else hi = mid - 1;
       }
-      const int g = *(volatile int32_t *)(p.dlist + lo);
+      g = *(volatile int32_t *)(p.dlist + lo);
       c = __ldg(p.seg_chunk0 + g) + (ci - *(volatile int64_t *)(p.dpref + lo));
       gs = __ldg(p.graph_s + g);
       c0 = __ldg(p.graph_col0 + g);
@@ -596,7 +680,7 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
         if (tc) {
 #pragma unroll
           for (int q = 0; q < U; ++q)
-            if (u[q] >= 0 && !((L.Cp[u[q] >> 5] >> (u[q] & 31)) & 1u)) u[q] = -1;
+            if (u[q] >= 0 && !changed(L.Mp, u[q])) u[q] = -1;
         }
 #pragma unroll
         for (int q = 0; q < U; ++q)
@@ -613,8 +697,7 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
       } else if (need) {  // only whether the row is active
 #pragma unroll
         for (int q = 0; q < U; ++q)
-          if (u[q] >= 0 && gather_ok(p, u[q], 0))
-            found |= ((L.Cp[u[q] >> 5] >> (u[q] & 31)) & 1u) != 0u;
+          if (u[q] >= 0 && gather_ok(p, u[q], 0)) found |= changed(L.Mp, u[q]);
       }
       need = open || (need && !PW && !found);
       if (more) {
@@ -627,9 +710,7 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
     // m_active
     uint32_t gdeg = 0;
     if (act) {
-      const unsigned long long deg =
-          whole ? (unsigned long long)len
-                : (unsigned long long)(__ldg(p.row_ptr + v + 1) - __ldg(p.row_ptr + v));
+      const unsigned long long deg = whole ? (uint32_t)len : p.deg_in[v];
       if constexpr (PW) {
         uint32_t mask = 0;
 #pragma unroll
@@ -640,14 +721,14 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
         L.rows += __popc(mask);
         for (; mask; mask &= mask - 1)
           L.work += deg * __popcll(valid_mask(__ffs(mask) - 1, p.s));
-      } else if (whole || !set_bit(L.Kc, v)) {
+      } else if (whole || !(mark(L.Mc, v, kClaimed) & kClaimed)) {
         L.mact += deg;
-        L.work += deg * (unsigned long long)gs;
+        if (SEG) L.work += deg * (unsigned long long)gs;
         ++L.rows;
         gdeg = (uint32_t)deg;
       }
     }
-    if (gm) {  // the rows of a chunk are one graph's
+    if (SEG && gm) {  // the rows of a chunk are one graph's
       const unsigned any = __ballot_sync(kFullMask, gdeg != 0u);
       if (any) {
         unsigned long long sum = gdeg;
@@ -687,10 +768,10 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
     bool app = false;
     if (gain) {
       if (whole) {
-        atomicOr(L.Cc + (v >> 5), 1u << (v & 31));
+        mark(L.Mc, v, kChanged);
         app = true;
       } else {
-        app = !set_bit(L.Cc, v);
+        app = !(mark(L.Mc, v, kChanged) & kChanged);
       }
     }
     if (__any_sync(kFullMask, gain)) {
@@ -699,10 +780,11 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
         if (__any_sync(kFullMask, acc[k] != 0ULL)) {
           const uint32_t n0 = __popc(transpose32((uint32_t)acc[k], L.lane));
           const uint32_t n1 = __popc(transpose32((uint32_t)(acc[k] >> 32), L.lane));
-          if (n0) atomicAdd(L.cnt + c0 + k * 64 + L.lane, n0);
-          if (n1) atomicAdd(L.cnt + c0 + k * 64 + 32 + L.lane, n1);
+          if (n0) count_add(L, c0 + k * 64 + L.lane, n0);
+          if (n1) count_add(L, c0 + k * 64 + 32 + L.lane, n1);
         }
-      if (L.scnt > kStage - 32) stage_spill(p, L);
+      if (L.scnt > kStage - 32) stage_spill<SEG>(p, L);
+      if (app) stage_degree<SEG>(p, L, p.deg_out[v], g);
       stage_row(L, v, app);
     }
   }
@@ -738,14 +820,13 @@ __device__ void list_dense(const Params &p, int cur) {
   }
 }
 
-template <int CW, bool PW>
-__global__ void __launch_bounds__(1024, 1)
+template <int CW, bool PW, bool SEG>
+__global__ void __launch_bounds__(kMaxThreads, 1)
     k_rounds(const __grid_constant__ Params p, const int32_t *seeds, const int32_t *seed_bit,
              int sp, int resume, int epoch) {
   extern __shared__ uint32_t dyn[];
   __shared__ Shared sh;
-  const bool smem_counts = p.ncols <= kResidentCounts;
-  uint32_t *scnt_s = smem_counts ? dyn : nullptr;
+  const bool smem_counts = p.ncols <= kResidentCounts;  // two rows of counters, by round parity
   Ctrl *ctrl = p.ctrl;
   ResidentCtl *rc = p.rctl;
   Lane L;
@@ -755,19 +836,22 @@ __global__ void __launch_bounds__(1024, 1)
   L.nwarps = (int64_t)gridDim.x * (blockDim.x >> 5);
   L.tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   L.nth = (int64_t)gridDim.x * blockDim.x;
-  L.stage = reinterpret_cast<int32_t *>(dyn + (smem_counts ? p.ncols : 0)) + L.wid * kStage;
+  L.stage = reinterpret_cast<int32_t *>(dyn + (smem_counts ? 2 * p.ncols : 0)) + L.wid * kStage;
   L.scnt = 0;
-  L.mact = L.work = L.scan = L.gath = L.items = 0;
-  L.rows = 0;
-  if (scnt_s)
-    for (int i = threadIdx.x; i < p.ncols; i += blockDim.x) scnt_s[i] = 0u;
+  L.od = L.ne = L.gacc = 0;
+  L.gcur = -1;
+  L.mact = L.work = 0;
+  L.rows = L.scan = L.gath = L.items = 0;
+  if (smem_counts)
+    for (int i = threadIdx.x; i < 2 * p.ncols; i += blockDim.x) dyn[i] = 0u;
   if (threadIdx.x == 0) {
-    sh.mact = sh.work = 0;
-    sh.rows = 0;
+    sh.mact = sh.work = sh.od = sh.ne = 0;
+    sh.rows = sh.staged = 0;
+    sh.bar = 0;
   }
   if (L.tid == 0) ctrl->bad_index = 0;
   auto none = [] {};
-  const int64_t kwords = PW ? (p.n + 3) / 4 : p.nbm;  // claim words
+  const int64_t mwords = (p.n + 15) / 16, kwords = (p.n + 3) / 4;  // marks, claim bytes
   int t;
   int64_t nF_old = 0;  // |F_{t-2}|
   int prev_dense = 0;  // round t was a sweep (its long rows are not in E)
@@ -788,18 +872,30 @@ __global__ void __launch_bounds__(1024, 1)
     }
     if ((words & 1) && L.tid == 0)
       p.X[words - 1] = p.D0[words - 1] = p.D1[words - 1] = p.D2[words - 1] = 0ULL;
-    for (int64_t i = L.tid; i < p.nbm; i += L.nth) p.C0[i] = p.C1[i] = p.C2[i] = 0u;
-    for (int64_t i = L.tid; i < kwords; i += L.nth) p.K0[i] = p.K1[i] = 0u;
+    for (int64_t i = L.tid; i < mwords; i += L.nth) p.C0[i] = p.C1[i] = p.C2[i] = 0u;
+    if constexpr (PW)
+      for (int64_t i = L.tid; i < kwords; i += L.nth) p.Kw0[i] = p.Kw1[i] = 0u;
+    // degrees as one 32-bit word a row (a row's columns are distinct, so < n):
+    // one access per claim or append instead of two row bounds
+    for (int64_t i = L.tid; i < p.n; i += L.nth)
+      p.deg_in[i] = (uint32_t)(__ldg(p.row_ptr + i + 1) - __ldg(p.row_ptr + i));
+    if (p.deg_out != p.deg_in)
+      for (int64_t i = L.tid; i < p.n; i += L.nth)
+        p.deg_out[i] = (uint32_t)(__ldg(p.out_ptr + i + 1) - __ldg(p.out_ptr + i));
     for (int64_t i = L.tid; i < (int64_t)p.ncols * 2 && i < (int64_t)p.ncols * p.row_cap; i += L.nth)
       p.counts[i] = 0u;
-    if (p.gfsum)
+    if constexpr (SEG)
       for (int64_t i = L.tid; i < 3LL * p.nseg; i += L.nth) p.gfsum[i] = 0ULL;
-    if (p.gmact)
+    if (SEG && p.gmact)
       for (int64_t i = L.tid; i < 2LL * p.nseg; i += L.nth) p.gmact[i] = 0ULL;
     if (L.tid == 0) ctrl->ndense = 0;
     if (L.tid < 2) p.rs[L.tid] = RoundStats{};
     if (L.tid < 3) rc->fp[L.tid] = rc->ne[L.tid] = 0ULL;
-    if (!grid_barrier(p, sh, none)) return;
+    if (!SEG && p.early_stop && L.tid < 3 * kAliveWords) {  // every seed starts alive
+      const int w = (int)L.tid % kAliveWords;
+      rc->alive[L.tid / kAliveWords][w] = L.tid < kAliveWords ? valid_mask(w, p.s) : 0ULL;
+    }
+    if (!grid_barrier<SEG>(p, sh, none)) return;
     for (int64_t base = L.warp * 32; base < sp; base += L.nwarps * 32) {
       const int64_t i = base + L.lane;
       unsigned long long od = 0;
@@ -813,13 +909,13 @@ __global__ void __launch_bounds__(1024, 1)
         }
         const int bit = seed_bit ? seed_bit[i] : (int)i;
         int col = (int)i;
-        if (p.node_graph) col = __ldg(p.graph_col0 + __ldg(p.node_graph + x)) + bit;
+        if (SEG) col = __ldg(p.graph_col0 + __ldg(p.node_graph + x)) + bit;
         red_or(p.X + (size_t)x * CW + (bit >> 6), 1ULL << (bit & 63));
         red_or(p.D0 + (size_t)x * CW + (bit >> 6), 1ULL << (bit & 63));
         atomicAdd(p.counts + col, 1u);
-        first = !set_bit(p.C0, x);
+        first = !(mark(p.C0, x, kChanged) & kChanged);
         if (first) od = (unsigned long long)(__ldg(p.out_ptr + x + 1) - __ldg(p.out_ptr + x));
-        if (p.gfsum && od) atomicAdd(p.gfsum + __ldg(p.node_graph + x), od);
+        if (SEG && od) atomicAdd(p.gfsum + __ldg(p.node_graph + x), od);
       }
       const unsigned mask = __ballot_sync(kFullMask, first);
       if (!mask) continue;
@@ -837,7 +933,7 @@ __global__ void __launch_bounds__(1024, 1)
       if (first) p.F0[bf + __popc(mask & ((1u << L.lane) - 1u))] = x;
       if (et) write_pieces(p.E, be + ex, x, ne, L.lane);
     }
-    if (!grid_barrier(p, sh, [&] { list_dense(p, 0); })) return;
+    if (!grid_barrier<SEG>(p, sh, [&] { list_dense(p, 0); })) return;
     t = 0;  // round 0 is complete
   } else {
     t = ctrl->t - 1;
@@ -847,23 +943,39 @@ __global__ void __launch_bounds__(1024, 1)
     // a new counts window: its first row and statistics slot
     for (int64_t i = L.tid; i < (int64_t)p.ncols * 2 && i < (int64_t)p.ncols * p.row_cap; i += L.nth)
       p.counts[i] = 0u;
-    if (p.gmact)
+    if (SEG && p.gmact)
       for (int64_t i = L.tid; i < 2LL * p.nseg; i += L.nth) p.gmact[i] = 0ULL;
     if (L.tid < 2) p.rs[L.tid] = RoundStats{};
-    if (!grid_barrier(p, sh, none)) return;
+    if (!grid_barrier<SEG>(p, sh, none)) return;
   }
   bool first_pass = resume != 0;  // round t's statistics are in the last window
   for (;;) {
     // round t is complete: what it left, the same in every block
+    // (one reader a block: every warp of the grid at one word would queue)
     if (threadIdx.x == 0) {
       sh.fp = *(volatile unsigned long long *)&rc->fp[t % 3];
       sh.ne_all = *(volatile unsigned long long *)&rc->ne[t % 3];
     }
     __syncthreads();
-    const int64_t nF = (int64_t)(sh.fp >> kFsumBits);
-    const int64_t fsum = (int64_t)(sh.fp & kFsumMask);
+    const unsigned long long fp = sh.fp;
     int64_t nE = (int64_t)sh.ne_all;
+    const int64_t nF = (int64_t)(fp >> kFsumBits);
+    const int64_t fsum = (int64_t)(fp & kFsumMask);
     const bool lead = blockIdx.x == 0 && threadIdx.x == 0;
+    // round t's counts leave the block here, while the next round starts: a
+    // block adds up to ncols words to the same few lines as every other, and
+    // at the end of the round the barrier would wait for that queue
+    if (smem_counts && !first_pass) {
+      uint32_t *cs = dyn + (t & 1) * p.ncols;
+      uint32_t *crow = p.counts + (size_t)(t - p.row_base) * (size_t)p.ncols;
+      for (int i = threadIdx.x; i < p.ncols; i += blockDim.x) {
+        const uint32_t c = cs[i];
+        if (c) {
+          atomicAdd(&crow[i], c);
+          cs[i] = 0u;
+        }
+      }
+    }
     if (lead && !first_pass) {
       RoundStats *r = p.rs + (t - p.row_base);
       r->changed = (unsigned long long)nF;
@@ -894,10 +1006,9 @@ __global__ void __launch_bounds__(1024, 1)
       break;
     }
     first_pass = false;
-    const bool dense = !p.gfsum && (p.direction == PG_DIR_DENSE ||
-                                    (p.direction == PG_DIR_AUTO &&
-                                     (double)fsum > (double)p.dense_threshold * (double)p.m));
-    const bool tc = p.test_adapt ? (double)fsum < kTestDensity * (double)p.m : p.test_changed != 0;
+    const bool dense = !SEG && (p.direction == PG_DIR_DENSE ||
+                                    (p.direction == PG_DIR_AUTO && fsum > p.dense_above));
+    const bool tc = p.test_adapt ? 2 * fsum < p.m : p.test_changed != 0;  // kTestDensity
     const int prev = t % 3;
     ++t;
     L.t = t;
@@ -905,16 +1016,18 @@ __global__ void __launch_bounds__(1024, 1)
     const int old = (t + 1) % 3;  // of round t-2, next of round t+1
     L.Dp = delta_buf(p, prev);
     L.Dc = delta_buf(p, L.cur);
-    L.Cp = changed_buf(p, prev);
-    L.Cc = changed_buf(p, L.cur);
-    L.Kc = (t & 1) ? p.K1 : p.K0;
+    L.Mp = mark_buf(p, prev);
+    L.Mc = mark_buf(p, L.cur);
+    L.Kc = (t & 1) ? p.Kw1 : p.Kw0;
     L.F = frontier_buf(p, L.cur);
     L.E = (t & 1) ? p.E1 : p.E;
-    L.pieces = p.gfsum || !dense;
-    L.cnt = scnt_s ? scnt_s : p.counts + (size_t)(t - p.row_base) * (size_t)p.ncols;
+    L.pieces = SEG || !dense;
+    uint32_t *scnt_s = smem_counts ? dyn + (t & 1) * p.ncols : nullptr;
+    L.cs = scnt_s ? (uint32_t)__cvta_generic_to_shared(scnt_s) : 0u;
+    L.cg = p.counts + (size_t)(t - p.row_base) * (size_t)p.ncols;
     const int32_t *Fp = frontier_buf(p, prev);
     const unsigned long long *Ep = (t & 1) ? p.E : p.E1;
-    if (prev_dense && !dense && !p.gfsum) {
+    if (!SEG && prev_dense && !dense) {
       // after a sweep: the long rows of its frontier, in pieces
       unsigned long long *E = (t & 1) ? p.E : p.E1;
       for (int64_t base = L.warp * 32; base < nF; base += L.nwarps * 32) {
@@ -929,32 +1042,18 @@ __global__ void __launch_bounds__(1024, 1)
         }
         if (__any_sync(kFullMask, ne != 0ULL)) warp_append_pieces(E, &rc->ne[prev], v, ne, L.lane);
       }
-      if (!grid_barrier(p, sh, none)) return;
+      if (!grid_barrier<SEG>(p, sh, none)) return;
       if (threadIdx.x == 0) sh.ne_all = *(volatile unsigned long long *)&rc->ne[prev];
       __syncthreads();
       nE = (int64_t)sh.ne_all;
     }
-    if (dense && p.early_stop) {  // bits that can still travel: round t-1's seeds
-      const int pr = t - 1 - p.row_base;  // < 0: the row left with the last window
-      const uint32_t *row = p.counts + (size_t)(pr < 0 ? 0 : pr) * (size_t)p.ncols;
-      for (int w = L.wid; w < CW; w += blockDim.x >> 5) {
-        const int i = w * 64 + L.lane;
-        const unsigned lo = __ballot_sync(kFullMask, i < p.s && (pr < 0 || ld_u32(row + i) != 0u));
-        const unsigned hi =
-            __ballot_sync(kFullMask, i + 32 < p.s && (pr < 0 || ld_u32(row + i + 32) != 0u));
-        if (L.lane == 0) sh.alive[w] = ((uint64_t)hi << 32) | lo;
-      }
-      __syncthreads();
-    }
-    if (dense || (p.dlist && *(volatile int32_t *)&ctrl->ndense > 0))
-      sweep_round<CW, PW>(p, L, tc, dense && p.early_stop ? sh.alive : nullptr);
-    if (!dense) push_round<CW, PW>(p, L, Fp, Ep, nF, nE);
-    // round t-2's buffers become round t+1's
+    // round t-2's buffers become round t+1's; from the last thread down, as
+    // the work below goes from the first warp up
     {
       const ulonglong2 z = make_ulonglong2(0ULL, 0ULL);
       const int32_t *Fo = frontier_buf(p, old);
       uint64_t *Do = delta_buf(p, old);
-      for (int64_t i = L.tid; i < nF_old; i += L.nth) {
+      for (int64_t i = L.nth - 1 - L.tid; i < nF_old; i += L.nth) {
         uint64_t *dr = Do + (size_t)Fo[i] * CW;
         if constexpr (CW == 1) {
           dr[0] = 0ULL;
@@ -963,28 +1062,46 @@ __global__ void __launch_bounds__(1024, 1)
           for (int k = 0; k < CW; k += 2) *reinterpret_cast<ulonglong2 *>(dr + k) = z;
         }
       }
-      uint32_t *Co = changed_buf(p, old);
-      for (int64_t i = L.tid; i < p.nbm; i += L.nth) Co[i] = 0u;
-      uint32_t *Kn = (t & 1) ? p.K0 : p.K1;
-      for (int64_t i = L.tid; i < kwords; i += L.nth) Kn[i] = 0u;
+      uint32_t *Mo = mark_buf(p, old);
+      for (int64_t i = L.tid; i < mwords; i += L.nth) Mo[i] = 0u;
+      if constexpr (PW) {
+        uint32_t *Kn = (t & 1) ? p.Kw0 : p.Kw1;
+        for (int64_t i = L.tid; i < kwords; i += L.nth) Kn[i] = 0u;
+      }
       const int nrow = t + 1 - p.row_base;  // row t+1 of the counts window
       if (nrow < p.row_cap)
         for (int64_t i = L.tid; i < p.ncols; i += L.nth) p.counts[(size_t)nrow * p.ncols + i] = 0u;
-      if (p.gmact)
+      if (SEG && p.gmact)
         for (int64_t i = L.tid; i < p.nseg; i += L.nth) p.gmact[(size_t)nrow * p.nseg + i] = 0ULL;
-      if (p.gfsum)
+      if constexpr (SEG)
         for (int64_t i = L.tid; i < p.nseg; i += L.nth) p.gfsum[(size_t)old * p.nseg + i] = 0ULL;
       if (lead) {
         p.rs[nrow] = RoundStats{};
         rc->fp[old] = 0ULL;
         rc->ne[old] = 0ULL;
+        if (!SEG && p.early_stop)
+          for (int w = 0; w < CW; ++w) rc->alive[old][w] = 0ULL;
       }
     }
-    round_flush(p, L, sh, scnt_s);
-    if (!grid_barrier(p, sh, [&] { list_dense(p, L.cur); })) return;
+    if (dense && p.early_stop) {  // bits that can still travel: round t-1's seeds
+      if (threadIdx.x < CW) sh.alive[threadIdx.x] = *(volatile unsigned long long *)&rc->alive[prev][threadIdx.x];
+      __syncthreads();
+    }
+    if (SEG ? p.dlist && *(volatile int32_t *)&ctrl->ndense > 0 : dense)
+      sweep_round<CW, PW, SEG>(p, L, tc, dense && p.early_stop ? sh.alive : nullptr);
+    if (!dense) push_round<CW, PW, SEG>(p, L, Fp, Ep, nF, nE);
+    round_flush<PW, SEG>(p, L, sh, scnt_s);
+    if (!grid_barrier<SEG>(p, sh, [&] { list_dense(p, L.cur); })) return;
     nF_old = nF;
     prev_dense = dense;
     dense_rounds += dense;
+  }
+  // every block has passed the last barrier once it gets here; the last one
+  // out leaves the barrier's words as the next launch needs them
+  if (threadIdx.x == 0 && atomicAdd(&rc->exited, 1u) == gridDim.x - 1) {
+    rc->arrive = 0u;
+    rc->gen = 0u;
+    rc->exited = 0u;
   }
   // work counters of the launch, on the slot of its last round
   unsigned long long s3[3] = {L.scan, L.gath, L.items};
@@ -1002,18 +1119,23 @@ __global__ void __launch_bounds__(1024, 1)
 
 }  // namespace
 
-ResidentFn resident_fn(int CW, bool pw) {
+template <int CW>
+static ResidentFn pick_resident(bool pw, bool seg) {
+  return seg ? &k_rounds<CW, false, true> : pw ? &k_rounds<CW, true, false> : &k_rounds<CW, false, false>;
+}
+
+ResidentFn resident_fn(int CW, bool pw, bool seg) {
   switch (CW) {
-    case 1: return pw ? &k_rounds<1, true> : &k_rounds<1, false>;
-    case 2: return pw ? &k_rounds<2, true> : &k_rounds<2, false>;
-    case 4: return pw ? &k_rounds<4, true> : &k_rounds<4, false>;
-    case 8: return pw ? &k_rounds<8, true> : &k_rounds<8, false>;
+    case 1: return pick_resident<1>(pw, seg);
+    case 2: return pick_resident<2>(pw, seg);
+    case 4: return pick_resident<4>(pw, seg);
+    case 8: return pick_resident<8>(pw, seg);
   }
   return nullptr;
 }
 
 size_t resident_smem(int ncols, int threads) {
-  return sizeof(uint32_t) * (size_t)(ncols <= kResidentCounts ? ncols : 0) +
+  return sizeof(uint32_t) * (size_t)(ncols <= kResidentCounts ? 2 * ncols : 0) +
          sizeof(int32_t) * (size_t)(threads / 32) * kStage;
 }
 

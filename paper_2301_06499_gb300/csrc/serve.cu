@@ -406,6 +406,7 @@ void worker(pg_server *srv, int k) {
   for (;;) {
     Job job;
     pg_graph *master = nullptr;
+    int busy = 0;
     {
       std::unique_lock<std::mutex> lk(srv->mu);
       srv->cv.wait(lk, [&] { return srv->stop || (!srv->queue.empty() && pick(srv, k, job)); });
@@ -424,7 +425,11 @@ void worker(pg_server *srv, int k) {
       srv->st.inflight_bytes = slots_total(srv);
       srv->st.peak_bytes = std::max(srv->st.peak_bytes, resident_total(srv) + slots_total(srv));
       master = srv->graphs.at(job.graph).g;
+      for (auto &sl : srv->slots) busy += sl->busy ? 1 : 0;
     }
+    // propagations that run side by side share the SMs: a resident round loop
+    // that asks for more than are free waits for the others to end
+    const int sms = busy > 1 ? std::max(1, sm_count() / busy) : 0;
     // outside the lock: the propagation
     pg_status rc = PG_OK;
     Split sp;
@@ -452,6 +457,7 @@ void worker(pg_server *srv, int k) {
       }
       if (rc == PG_OK) {
         const int32_t maxr = (int32_t)std::min<int64_t>(master->n - 1, 0x3FFFFFFF);
+        view->sms = sms;
         rc = propagate_columns(view, seeds.data(), (int32_t)seeds.size(), maxr, &split_window,
                                &sp, &T, &srv->cfg.opt, me.stream, &pst);
       }
@@ -488,6 +494,7 @@ void worker(pg_server *srv, int k) {
         for (size_t gk = 0, i = 0; gk < job.graphs.size(); ++gk)
           for (int32_t b = 0; b < gs[gk]; ++b, ++i) seeds[i] += (int32_t)u.v0[gk];
         u.g->ext_ws = &me.ws;
+        u.g->sms = sms;
         int32_t smax = 0;
         for (int32_t x : gs) smax = std::max(smax, x);
         rc = propagate_batch_group(u.g, seeds.data(), bits.data(), (int32_t)seeds.size(),

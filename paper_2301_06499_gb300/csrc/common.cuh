@@ -152,6 +152,7 @@ struct Params {
                         // of copy k maps to k*perm_n + perm[x])
   ResidentCtl *rctl;    // resident loop (else null)
   uint32_t *deg_in, *deg_out;  // resident loop: degrees (the same array for symmetric graphs)
+  int32_t sort_seeds;   // resident loop: bits of rows of 8 words placed by the seeds' degree
   int64_t dense_above;  // resident loop: a full sweep when the frontier's out-arcs pass this
   int32_t col_quads;    // resident loop: out_col is 16-byte aligned
   int32_t row_base;     // resident loop: round in row 0 of the counts window

@@ -1107,10 +1107,11 @@ using PullFn = void (*)(Params);
 // 1.87 against 2.05 ms, 1024^2 grid 40.5 against 47.3 ms.
 constexpr int kResidentThreads = 512;
 constexpr int kResidentCounts = 8192;
+constexpr int kResidentSorted = 512;  // most seeds whose bits are placed by degree
 constexpr int kResidentRow = 32;      // out-arcs of a frontier row that one group of lanes pushes
 constexpr int kResidentPiece = 128;   // out-arcs of a longer row per warp
 using ResidentFn = void (*)(Params, const int32_t *, const int32_t *, int, int, int);
-ResidentFn resident_fn(int CW, bool pw, bool seg);
+ResidentFn resident_fn(int CW, bool pw, bool seg, bool pair = false);
 size_t resident_smem(int ncols, int threads);
 // Push rounds as a kernel of their own (k_push<CW, PW>, push.cu): 8-word
 // rows, PROPAGATE-S passes as words and packed batches; it returns at once in

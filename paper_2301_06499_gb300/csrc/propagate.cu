@@ -955,14 +955,15 @@ struct BatchSeg {
 // as a part of all arcs, where the caller keeps the default. A pushed arc costs
 // several swept ones, but a sweep of a graph without long rows (grids, road
 // networks, uniform random graphs) costs its whole latency: 1024^2 grid
-// (s = 128) 37.1 ms a call at 0.2 against 51.1 at 0.05, ER within 1% either
-// way. With hubs the sends of one long row collide: R-MAT 22 (s = 256) 1.89 ms
-// at 0.05 against 2.14 at 0.2, R-MAT 18 (s = 100) 0.57 against 0.69.
+// (s = 128) 37.2 ms a call at 0.2 against 52.1 at 0.05, ER within 5% either
+// way. With hubs: R-MAT 26 (s = 512, a round of 7.6% of the arcs) 44.5 ms at
+// 0.08 against 49.8 at 0.05; R-MAT 20 (s = 400) 0.83 ms at 0.08 against 0.95
+// at 0.1; R-MAT 18 (s = 100) 0.57 against 0.62 at 0.2.
 constexpr int64_t kEvenDegree = 64;
 
 static double resident_threshold(const pg_graph *g, const pg_options &o) {
   if (o.dense_threshold > 0 && o.dense_threshold != 0.05f) return (double)o.dense_threshold;
-  return g->max_degree <= kEvenDegree ? 0.2 : (double)0.05f;
+  return g->max_degree <= kEvenDegree ? 0.2 : 0.08;
 }
 
 // Threads per block of a resident round loop of one block per SM: about a warp
@@ -984,8 +985,8 @@ static void resident_smem_optin() {
   std::lock_guard<std::mutex> lk(mu);
   if (dev < 64 && (done >> dev) & 1ULL) return;
   for (int cw : {1, 2, 4, 8})
-    for (int kind = 0; kind < 3; ++kind)
-      cudaFuncSetAttribute((const void *)resident_fn(cw, kind == 1, kind == 2),
+    for (int kind = 0; kind < (cw == 8 ? 5 : 3); ++kind)
+      cudaFuncSetAttribute((const void *)resident_fn(cw, kind == 1 || kind == 4, kind == 2, kind > 2),
                            cudaFuncAttributeMaxDynamicSharedMemorySize,
                            (int)resident_smem(kResidentCounts, kResidentThreads));
   if (dev < 64) done |= 1ULL << dev;
@@ -1003,11 +1004,14 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   }
   p.rctl = (ResidentCtl *)w.rctl.p;
   resident_smem_optin();
-  const ResidentFn fn = resident_fn(pl.CW, pl.pw, batch);
+  const bool pair = pl.CW == 8 && !batch && p.early_stop;
+  const ResidentFn fn = resident_fn(pl.CW, pl.pw, batch, pair);
   // the SMs given to this graph (propagations that run side by side share
   // them: a cooperative launch waits until all its blocks fit), else all
   const int blocks = cl.g->sms > 0 ? std::min(cl.g->sms, sm_count()) : sm_count();
   const int threads = resident_threads(p.n, blocks);
+  // a seed's bit is the loop's own business unless bits are passes
+  p.sort_seeds = pair && !pl.pw && sp > 256 && sp <= kResidentSorted;
   const size_t smem = resident_smem(p.ncols, threads);
   const int32_t *seeds = (const int32_t *)w.seeds.p;
   const int32_t *bits = batch ? (const int32_t *)w.seed_bits.p : nullptr;

@@ -33,10 +33,14 @@
 // as k_pull does, with its early stop.
 //
 // Measured per call, round by round (with dense rounds that stop early) and
-// resident: ER 10^3 (s = 64) 214 -> 136 us, ER 10^4 (s = 64) 282 -> 209 us,
-// 1024^2 grid (s = 128, ~2,050 rounds) 82.7 -> 55.8 ms, R-MAT 22 (s = 256)
-// 2.23 -> 1.91 ms, R-MAT 26 (s = 512) 54.9 -> 46.7 ms, 30 packed graphs
-// 33.6 -> 18.6 ms.
+// here: ER 10^3 (s = 64) 215 -> 128 us, ER 10^4 (s = 64) 288 -> 160 us,
+// 1024^2 grid (s = 128, ~2,050 rounds) 83 -> 36.5 ms, R-MAT 22 (s = 256)
+// 2.23 -> 1.70 ms, R-MAT 26 (s = 512) 54.9 -> 42 ms, 30 packed graphs
+// 33.6 -> 16.3 ms. What bounds it now: a round of little work is five
+// dependent accesses, two block-wide steps and the barrier, 6 to 7 us; heavy
+// pushes the L2's atomics (about 25 per ns on spread addresses), which is why
+// marks are loaded before they are set; heavy sweeps the gathers a thread's
+// registers can hold in flight.
 //
 // Every wait at the barrier is bounded; on expiry the call returns
 // PG_ETIMEOUT. The blocks are co-resident by the cooperative launch.
@@ -123,6 +127,8 @@ struct Shared {
   unsigned long long mact, work;
   uint32_t rows, staged;
   uint64_t alive[kAliveWords];
+  uint16_t col[kResidentSorted];   // count column of each bit (p.sort_seeds)
+  uint16_t place[kResidentSorted]; // bit of each seed
   unsigned long long fp, ne_all;
   uint32_t bar;  // barriers this block has arrived at
   int last;      // this block arrived last
@@ -410,49 +416,61 @@ __device__ __forceinline__ uint32_t claim_passes(uint32_t *Kb, int64_t v, uint32
 }
 
 // ------------------------------------------------------------ sparse rounds
-// A lane holds at most two words of a row: rows of 4 and 8 words take 2 and 4
-// lanes, so that four out-arcs a lane fit the registers at every width. The
-// loads of the four arcs are issued together, then their atomics, then the
-// atomics and loads that depend on those: a frontier row of four arcs costs
-// five dependent accesses, not five per arc.
+// A lane takes four out-arcs of a frontier row together: their loads, then
+// their signature atomics, then their marks are under way at once, so that a
+// row of four arcs costs five dependent accesses, not five per arc. Of a row's
+// words only the pairs with new bits are sent, one pair after another: a
+// sparse round's delta holds a bit or two, and rows of 8 words then cost what
+// rows of 2 do. (Four lanes a row, two words each, took 9.6 ms for 105 M hub
+// arcs of R-MAT 26 at s = 512 and 2.5 ms for its 10 M short rows.)
 template <int CW, bool PW, bool SEG>
 __device__ __forceinline__ void push_round(const Params &p, Lane &L, const int32_t *Fp,
                                            const unsigned long long *Ep, int64_t nF, int64_t nE) {
-  constexpr int UNR = 4;                  // out-arcs a lane handles together
-  constexpr int WL = CW <= 2 ? CW : 2;    // words of a row per lane
-  constexpr int SUB = CW / WL;            // lanes per row
-  constexpr int ROWS = 32 / SUB;          // rows per warp
-  const int sub = L.lane % SUB, r = L.lane / SUB, w0 = sub * WL;
+  constexpr int UNR = 4;                // out-arcs a lane handles together
+  constexpr int WL = CW <= 2 ? CW : 2;  // words sent together
+  constexpr int PAIRS = CW / WL;
   // a small frontier spreads each row's arcs over more lanes, so that its
   // rows of up to kBigRow arcs take one step
-  int gl = 0;  // log2 of the lane groups per row
-  while (gl < 3 && (nF * SUB << (gl + 1)) <= L.nth) ++gl;
-  const int rows = ROWS >> gl;  // rows per warp
+  int gl = 0;  // log2 of the lanes per row
+  while (gl < 3 && (nF << (gl + 1)) <= L.nth) ++gl;
+  const int rows = 32 >> gl;  // rows per warp
   const int64_t groups = (nF + rows - 1) / rows;
   const unsigned long long *gfp =
       SEG ? p.gfsum + (size_t)((L.t + 2) % 3) * (size_t)p.nseg : nullptr;
-  for (int64_t it = L.warp; it < groups + nE; it += L.nwarps) {
-    int32_t u = -1;
-    int64_t ob = 0, oe = 0;
-    int stride = 1;
+  // a degree is wanted once per claimed row; while all of them sit in L2 it is
+  // fetched with the signature, else after the claim (one access in eight on
+  // the hub rows of R-MAT 26)
+  const bool deg_now = p.n <= (1 << 22);
+  // row and arcs of an item: fetched for the next item ahead of this one's work
+  auto item = [&](int64_t it, int32_t &u, int64_t &ob, int64_t &oe) {
+    u = -1;
+    ob = oe = 0;
     if (it < groups) {
-      const int64_t i = it * rows + (r >> gl);
-      stride = 1 << gl;
+      const int64_t i = it * rows + (L.lane >> gl);
       if (i < nF) {
         u = Fp[i];
         ob = __ldg(p.out_ptr + u);
         oe = __ldg(p.out_ptr + u + 1);
         if (oe - ob > kBigRow) oe = ob;  // in pieces, below
-        ob += r & (stride - 1);
+        ob += L.lane & ((1 << gl) - 1);
       }
-    } else {
+    } else if (it < groups + nE) {
       const unsigned long long e = Ep[it - groups];
       u = (int32_t)(e >> 32);
       const int64_t b0 = __ldg(p.out_ptr + u) + (int64_t)(e & 0xFFFFFFFFULL) * kBigPiece;
       oe = min(__ldg(p.out_ptr + u + 1), b0 + kBigPiece);
-      ob = b0 + r;
-      stride = ROWS;
+      ob = b0 + L.lane;
     }
+  };
+  int32_t u_next;
+  int64_t ob_next, oe_next;
+  item(L.warp, u_next, ob_next, oe_next);
+  for (int64_t it = L.warp; it < groups + nE; it += L.nwarps) {
+    const int32_t u = u_next;
+    int64_t ob = ob_next, oe = oe_next;
+    const bool piece = it >= groups;  // 32 lanes on one long row: the same delta
+    const int stride = piece ? 32 : 1 << gl;
+    item(it + L.nwarps, u_next, ob_next, oe_next);
     int gs = p.s, c0 = 0, g = 0;
     unsigned long long *gm = nullptr;
     if (SEG && u >= 0) {
@@ -463,20 +481,25 @@ __device__ __forceinline__ void push_round(const Params &p, Lane &L, const int32
       c0 = __ldg(p.graph_col0 + g);
       if (p.gmact) gm = p.gmact + (size_t)(L.t - p.row_base) * (size_t)p.nseg + g;
     }
-    uint64_t d[WL];
+    uint64_t d[CW];
 #pragma unroll
-    for (int k = 0; k < WL; ++k) d[k] = 0ULL;
+    for (int k = 0; k < CW; ++k) d[k] = 0ULL;
     if (ob < oe && gather_ok(p, u, CW - 1)) {
-      ld_row<WL>(d, L.Dp + (size_t)u * CW + w0);
-      if (sub == 0) {
-        ++L.items;
-        ++L.gath;
-      }
+      ld_row<CW>(d, L.Dp + (size_t)u * CW);
+      ++L.items;
+      ++L.gath;
+    }
+    uint32_t pairs = 0;  // the pairs of words with new bits
+#pragma unroll
+    for (int j = 0; j < PAIRS; ++j) {
+      uint64_t any = 0;
+#pragma unroll
+      for (int k = 0; k < WL; ++k) any |= d[j * WL + k];
+      if (any) pairs |= 1u << j;
     }
     while (__any_sync(kFullMask, ob < oe)) {
       int32_t v[UNR];
-      uint64_t x[UNR][WL];
-      uint32_t deg[UNR], bits = 0;
+      uint32_t deg[UNR], mk[UNR];
       if (stride == 1 && p.col_quads && (ob & ~3LL) + 8 <= p.m) {
         // a row's next four arcs: the two 16-byte quads that hold them
         int4 lo = make_int4(-1, -1, -1, -1), hi = lo;
@@ -502,81 +525,135 @@ __device__ __forceinline__ void push_round(const Params &p, Lane &L, const int32
       for (int q = 0; q < UNR; ++q) {
         if (v[q] >= 0 && !gather_ok(p, v[q], CW - 1)) v[q] = -1;
         deg[q] = 0;
-#pragma unroll
-        for (int k = 0; k < WL; ++k) x[q][k] = ~0ULL;
+        mk[q] = ~0u;
         if (v[q] >= 0) {
-          ld_row<WL>(x[q], p.X + (size_t)v[q] * CW + w0);
-          if (sub == 0) {
-            ++L.scan;
-            deg[q] = p.deg_in[v[q]];
-          }
+          ++L.scan;
+          mk[q] = ld_u32(L.Mc + (v[q] >> 4));  // an atomic only for a mark not seen set
+          if (deg_now) deg[q] = p.deg_in[v[q]];
         }
       }
-      // rows with a zero bit left (PW: per pass, and only passes sent to),
-      // over the row's lanes
-#pragma unroll
-      for (int q = 0; q < UNR; ++q)
+      uint32_t gain = 0, room = 0;  // by arc; PW: room by arc and word
+      uint32_t left = pairs;
+      do {
+        const int j = left ? __ffs(left) - 1 : 0;
+        const bool on = left != 0u;
+        left &= left - 1;
+        const int w0 = j * WL;
+        uint64_t dj[WL], x[UNR][WL], old[UNR][WL];
 #pragma unroll
         for (int k = 0; k < WL; ++k) {
-          const bool room = (x[q][k] | ~valid_mask(w0 + k, gs)) != ~0ULL;
-          if constexpr (PW) {
-            if (room && d[k]) bits |= 1u << (8 * q + w0 + k);
-          } else {
-            if (room) bits |= 1u << q;
+          dj[k] = d[k];
+#pragma unroll
+          for (int i = 1; i < PAIRS; ++i)
+            if (j == i) dj[k] = d[i * WL + k];
+        }
+#pragma unroll
+        for (int q = 0; q < UNR; ++q) {
+#pragma unroll
+          for (int k = 0; k < WL; ++k) x[q][k] = ~0ULL;
+          if (on && v[q] >= 0) ld_row<WL>(x[q], p.X + (size_t)v[q] * CW + w0);
+        }
+#pragma unroll
+        for (int q = 0; q < UNR; ++q)
+#pragma unroll
+          for (int k = 0; k < WL; ++k) {
+            // a zero bit left (PW: per pass, and only passes sent to)
+            if ((x[q][k] | ~valid_mask(w0 + k, gs)) != ~0ULL) {
+              if constexpr (PW) {
+                if (dj[k]) room |= 1u << (8 * q + w0 + k);
+              } else {
+                room |= 1u << q;
+              }
+            }
+            // the bits the row lacks: all atomics under way at once
+            x[q][k] = dj[k] & ~x[q][k];
+            old[q][k] = 0ULL;
+            if (x[q][k])
+              old[q][k] = (uint64_t)atomicOr(
+                  reinterpret_cast<unsigned long long *>(p.X + (size_t)v[q] * CW + w0 + k),
+                  (unsigned long long)x[q][k]);
           }
-        }
+        // new bits: each has this lane as its only finder
 #pragma unroll
-      for (int off = SUB >> 1; off > 0; off >>= 1) bits |= __shfl_xor_sync(kFullMask, bits, off);
-      // the bits each row lacks: all atomics under way at once
-      uint64_t old[UNR][WL];
+        for (int q = 0; q < UNR; ++q)
 #pragma unroll
-      for (int q = 0; q < UNR; ++q)
-#pragma unroll
-        for (int k = 0; k < WL; ++k) {
-          x[q][k] = v[q] >= 0 ? d[k] & ~x[q][k] : 0ULL;
-          old[q][k] = 0ULL;
-          if (x[q][k])
-            old[q][k] = (uint64_t)atomicOr(
-                reinterpret_cast<unsigned long long *>(p.X + (size_t)v[q] * CW + w0 + k),
-                (unsigned long long)x[q][k]);
-        }
-      // new bits: each has this lane as its only finder
-      uint32_t gain = 0;
-#pragma unroll
-      for (int q = 0; q < UNR; ++q)
-#pragma unroll
-        for (int k = 0; k < WL; ++k) {
-          x[q][k] &= ~old[q][k];
-          if (x[q][k]) {
-            red_or(L.Dc + (size_t)v[q] * CW + w0 + k, x[q][k]);
-            gain |= 1u << q;
+          for (int k = 0; k < WL; ++k) {
+            x[q][k] &= ~old[q][k];
+            if (x[q][k]) {
+              red_or(L.Dc + (size_t)v[q] * CW + w0 + k, x[q][k]);
+              gain |= 1u << q;
+            }
           }
-        }
+        if (piece) {  // one delta for the warp: its bits counted over the lanes
 #pragma unroll
-      for (int off = SUB >> 1; off > 0; off >>= 1) gain |= __shfl_xor_sync(kFullMask, gain, off);
+          for (int k = 0; k < WL; ++k) {
+            uint64_t any = 0;
+#pragma unroll
+            for (int q = 0; q < UNR; ++q) any |= x[q][k];
+            if (!__any_sync(kFullMask, any != 0ULL)) continue;
+            uint64_t m = __shfl_sync(kFullMask, dj[k], 0);  // the piece's first lane has an arc
+            while (m) {
+              const int bit = __ffsll((long long)m) - 1;
+              m &= m - 1;
+              uint32_t n = 0;
+#pragma unroll
+              for (int q = 0; q < UNR; ++q) n += (uint32_t)(x[q][k] >> bit) & 1u;
+              n = __reduce_add_sync(kFullMask, n);
+              if (L.lane == 0 && n) count_add(L, c0 + (w0 + k) * 64 + bit, n);
+            }
+          }
+        } else {
+#pragma unroll
+          for (int q = 0; q < UNR; ++q)
+#pragma unroll
+            for (int k = 0; k < WL; ++k) count_bits(L, c0, w0 + k, x[q][k]);
+        }
+      } while (__any_sync(kFullMask, left != 0u));
+      if constexpr (!PW && PAIRS > 1) {
+        // full in every word sent: the others decide whether the row is active
+#pragma unroll
+        for (int q = 0; q < UNR; ++q)
+          if (v[q] >= 0 && !((room >> q) & 1u)) {
+            uint64_t y[CW];
+            ld_row<CW>(y, p.X + (size_t)v[q] * CW);
+            bool full = true;
+#pragma unroll
+            for (int k = 0; k < CW; ++k) full &= (y[k] | ~valid_mask(k, gs)) == ~0ULL;
+            if (!full) room |= 1u << q;
+          }
+      }
       // the claim and the place in F_t, for rows with room
-      uint32_t mk[UNR], od[UNR];
+      uint32_t od[UNR];
 #pragma unroll
       for (int q = 0; q < UNR; ++q) {
-        mk[q] = ~0u;
-        od[q] = deg[q];
+        od[q] = 0;
         const bool gq = (gain >> q) & 1u;
-        if (sub == 0 && (PW ? gq : ((bits >> q) & 1u) != 0u)) {
-          mk[q] = mark_word(L.Mc, v[q], gq ? kClaimed | kChanged : kClaimed);
-          if (gq && p.deg_out != p.deg_in) od[q] = p.deg_out[v[q]];
+        const uint32_t want = (gq ? kChanged : 0u) | (!PW && ((room >> q) & 1u) ? kClaimed : 0u);
+        if (!want) mk[q] = ~0u;
+        if (want & ~(mk[q] >> ((v[q] & 15) * 2))) {
+          mk[q] = mark_word(L.Mc, v[q], want);
+          if (deg_now && gq && p.deg_out != p.deg_in) od[q] = p.deg_out[v[q]];
         }
       }
-#pragma unroll
-      for (int q = 0; q < UNR; ++q)
-#pragma unroll
-        for (int k = 0; k < WL; ++k) count_bits(L, c0, w0 + k, x[q][k]);
 #pragma unroll
       for (int q = 0; q < UNR; ++q) {
         mk[q] >>= (v[q] & 15) * 2;
+        if (!deg_now) {
+          const bool app = ((gain >> q) & 1u) && !(mk[q] & kChanged);
+          if (v[q] >= 0 && (PW ? ((room >> (8 * q)) & 0xFFu) != 0u : !(mk[q] & kClaimed)))
+            deg[q] = p.deg_in[v[q]];
+          if (app) od[q] = p.deg_out[v[q]];
+        } else if (p.deg_out == p.deg_in) {
+          od[q] = deg[q];
+        }
+      }
+      if (L.scnt > kStage - 32 * UNR) stage_spill<SEG>(p, L);
+#pragma unroll
+      for (int q = 0; q < UNR; ++q) {
         if constexpr (PW) {
-          uint32_t m = (bits >> (8 * q)) & 0xFFu;
-          if (sub == 0 && m) m = claim_passes(L.Kc, v[q], m);
-          if (sub == 0 && m) {
+          uint32_t m = (room >> (8 * q)) & 0xFFu;
+          if (m) m = claim_passes(L.Kc, v[q], m);
+          if (m) {
             L.mact += (unsigned long long)deg[q] * __popc(m);
             L.rows += __popc(m);
             for (; m; m &= m - 1)
@@ -588,11 +665,7 @@ __device__ __forceinline__ void push_round(const Params &p, Lane &L, const int32
           ++L.rows;
           if (SEG && gm) atomicAdd(gm, (unsigned long long)deg[q]);
         }
-      }
-      if (L.scnt > kStage - UNR * ROWS) stage_spill<SEG>(p, L);
-#pragma unroll
-      for (int q = 0; q < UNR; ++q) {
-        const bool app = ((gain >> q) & 1u) && !(mk[q] & kChanged);  // mk is set on sub 0
+        const bool app = ((gain >> q) & 1u) && !(mk[q] & kChanged);
         if (app) stage_degree<SEG>(p, L, od[q], g);
         stage_row(L, v[q], app);
       }
@@ -605,78 +678,125 @@ __device__ __forceinline__ void push_round(const Params &p, Lane &L, const int32
 // The sweep of pull_dense (kernels.cuh) with its early stop, finishing each
 // row on the spot: new bits go to X and D of this round and are counted by a
 // 32 x 32 bit transpose per word and half.
-template <int CW, bool PW, bool SEG>
+//
+// PAIR (rows of 8 words, graphs of kEarlyStopArcs arcs and more): a lane holds
+// four words of a row (one 32-byte sector), a pair of lanes the row, and a
+// warp takes a chunk in two halves. The pair's gathers of a neighbour are one
+// L1 access instead of two, eight arcs a lane fit the registers, and each lane
+// stops at the arc where its own half can gain nothing more: R-MAT 20 (s =
+// 400) 996 -> 826 us a call. Smaller graphs wait for the two halves in turn
+// (900^2 grid, s = 500: 101 -> 120 ms), so a lane takes the whole row there.
+template <int CW, bool PW, bool SEG, bool PAIR>
 __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
                                             const uint64_t *alive) {
-  constexpr int U = CW <= 4 && !SEG ? 8 : 4;
-  constexpr bool kPipe = CW <= 4;  // at 8 words the registers are not there
-  const size_t Wp = CW;
+  constexpr int SUB = PAIR ? 2 : 1;       // lanes per row
+  constexpr int U = SEG || CW / SUB > 4 ? 4 : 8;  // arcs a lane gathers together
+  constexpr int WL = CW / SUB;            // words per lane
+  constexpr int RPW = 32 / SUB;           // rows per warp
+  const int sub = L.lane % SUB, w0 = sub * WL;
   const int nd = SEG ? *(volatile int32_t *)&p.ctrl->ndense : 0;
-  const int64_t nchunks = SEG ? *(volatile int64_t *)(p.dpref + nd) : p.sell_chunks;
-  for (int64_t ci = L.warp; ci < nchunks; ci += L.nwarps) {
-    int64_t c = ci;
-    int gs = p.s, c0 = 0, g = 0;
-    unsigned long long *gm = nullptr;
-    if constexpr (SEG) {  // the chunks of the graphs in a full sweep
+  const int64_t nunits = SUB * (SEG ? *(volatile int64_t *)(p.dpref + nd) : p.sell_chunks);
+  // a chunk's graph and place: all chunks in order, or (a packed batch) those
+  // of the graphs in a full sweep
+  auto chunk_at = [&](int64_t ci, int &g) -> int64_t {
+    if constexpr (!SEG) {
+      g = 0;
+      return ci;
+    } else {
       int lo = 0, hi = nd - 1;  // the last k with dpref[k] <= ci
       while (lo < hi) {
         const int mid = (lo + hi + 1) >> 1;
         if (*(volatile int64_t *)(p.dpref + mid) <= ci) lo = mid; else hi = mid - 1;
       }
       g = *(volatile int32_t *)(p.dlist + lo);
-      c = __ldg(p.seg_chunk0 + g) + (ci - *(volatile int64_t *)(p.dpref + lo));
+      return __ldg(p.seg_chunk0 + g) + (ci - *(volatile int64_t *)(p.dpref + lo));
+    }
+  };
+  // the next unit's descriptor is fetched when a unit starts, its first
+  // columns when the unit ends
+  int g_next = 0, clen_next = 0;
+  int64_t off_next = 0;
+  ulonglong2 it_next = make_ulonglong2(0ULL, 0ULL);
+  int32_t u_next[U];
+  auto descriptor = [&](int64_t ui) {
+    it_next = make_ulonglong2(0ULL, 0ULL);
+    clen_next = 0;
+    if (ui < nunits) {
+      const int64_t c = chunk_at(ui / SUB, g_next);
+      const int r = (int)(ui % SUB) * RPW + L.lane / SUB;  // row of the chunk
+      it_next = __ldg(p.sell_items + c * 32 + r);
+      clen_next = __ldg(p.sell_len + c);
+      off_next = __ldg(p.sell_off + c) + r;
+    }
+  };
+  auto first_columns = [&]() {
+    const int len = (int)(it_next.y & 0x7FFFFFFFULL);
+    const int32_t *cc = p.sell_col + off_next;
+#pragma unroll
+    for (int q = 0; q < U; ++q) u_next[q] = q < len ? __ldg(cc + 32LL * q) : -1;
+  };
+  descriptor(L.warp);
+  first_columns();
+  for (int64_t ui = L.warp; ui < nunits; ui += L.nwarps) {
+    int gs = p.s, c0 = 0;
+    const int g = g_next;
+    unsigned long long *gm = nullptr;
+    if constexpr (SEG) {
       gs = __ldg(p.graph_s + g);
       c0 = __ldg(p.graph_col0 + g);
       if (p.gmact) gm = p.gmact + (size_t)(L.t - p.row_base) * (size_t)p.nseg + g;
     }
-    const ulonglong2 it = p.sell_items[c * 32 + L.lane];
-    const int clen = __ldg(p.sell_len + c);
-    const int32_t *cc = p.sell_col + __ldg(p.sell_off + c) + L.lane;
+    const ulonglong2 it = it_next;
+    const int clen = clen_next;
+    const int32_t *cc = p.sell_col + off_next;
     const int32_t v = (int32_t)(it.y >> 32);
     const bool whole = (it.y & 0x80000000ULL) != 0ULL;
     const int len = (int)(it.y & 0x7FFFFFFFULL);
-    uint64_t own[CW], acc[CW];
+    uint64_t own[WL], acc[WL];
 #pragma unroll
-    for (int k = 0; k < CW; ++k) {
+    for (int k = 0; k < WL; ++k) {
       own[k] = ~0ULL;
       acc[k] = 0ULL;
     }
-    if (len > 0) ld_row<CW>(own, p.X + (size_t)v * Wp);
+    if (len > 0) ld_row<WL>(own, p.X + (size_t)v * CW + w0);
     int32_t u[U];
 #pragma unroll
-    for (int q = 0; q < U; ++q) u[q] = q < len ? __ldg(cc + 32LL * q) : -1;
+    for (int q = 0; q < U; ++q) u[q] = u_next[q];
+    descriptor(ui + L.nwarps);
+    auto pair_any = [&](bool x) {
+      return SUB == 1 ? x : (__shfl_xor_sync(kFullMask, (int)x, 1) != 0) || x;
+    };
     auto can_gain = [&]() {
       uint64_t r = 0;
 #pragma unroll
-      for (int k = 0; k < CW; ++k) {
-        const uint64_t lim = alive ? alive[k] : valid_mask(k, gs);
+      for (int k = 0; k < WL; ++k) {
+        const uint64_t lim = alive ? alive[w0 + k] : valid_mask(w0 + k, gs);
         r |= lim & ~(own[k] | acc[k]);
-        if (PW && !acc[k] && lim && (own[k] | ~valid_mask(k, p.s)) != ~0ULL) r |= 1ULL;
+        if (PW && !acc[k] && lim && (own[k] | ~valid_mask(w0 + k, p.s)) != ~0ULL) r |= 1ULL;
       }
       return r != 0ULL;
     };
     bool act = false;  // a zero bit left
 #pragma unroll
-    for (int k = 0; k < CW; ++k) act |= (own[k] | ~valid_mask(k, gs)) != ~0ULL;
+    for (int k = 0; k < WL; ++k) act |= (own[k] | ~valid_mask(w0 + k, gs)) != ~0ULL;
+    act = pair_any(act);
     bool open = act && can_gain();
     bool found = false;  // an in-neighbour changed
     bool need = PW ? open : act;
     for (int k0 = 0; k0 < clen; k0 += U) {
       if (!__any_sync(kFullMask, need)) break;
-      if (!kPipe && k0 > 0) {
-#pragma unroll
-        for (int q = 0; q < U; ++q)
-          u[q] = (need && k0 + q < len) ? __ldg(cc + 32LL * (k0 + q)) : -1;
-      }
       int32_t un[U];
-      const bool more = kPipe && k0 + U < clen;
+      const bool more = k0 + U < clen;
       if (more) {
 #pragma unroll
         for (int q = 0; q < U; ++q)
           un[q] = (need && k0 + U + q < len) ? __ldg(cc + 32LL * (k0 + U + q)) : -1;
       }
-      if (need) L.scan += (uint32_t)max(0, min(U, len - k0));
-      if (open) {
+      if (need && sub == 0) L.scan += (uint32_t)max(0, min(U, len - k0));
+      // (a pair gathers together until it has seen a change)
+      const bool pair_open = pair_any(open);  // every lane takes part in the exchange
+      const bool gather = open || (!PW && need && pair_open);
+      if (gather) {
         if (tc) {
 #pragma unroll
           for (int q = 0; q < U; ++q)
@@ -685,37 +805,43 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
 #pragma unroll
         for (int q = 0; q < U; ++q)
           if (u[q] >= 0 && gather_ok(p, u[q], CW - 1)) {
-            uint64_t d[CW];
-            ld_row<CW>(d, L.Dp + (size_t)u[q] * Wp);
+            uint64_t d[WL];
+            ld_row<WL>(d, L.Dp + (size_t)u[q] * CW + w0);
 #pragma unroll
-            for (int k = 0; k < CW; ++k) acc[k] |= d[k];
-            ++L.gath;
+            for (int k = 0; k < WL; ++k) acc[k] |= d[k];
+            if (sub == 0) ++L.gath;
           }
 #pragma unroll
-        for (int k = 0; k < CW; ++k) found |= acc[k] != 0ULL;
+        for (int k = 0; k < WL; ++k) found |= acc[k] != 0ULL;
         open = can_gain();
       } else if (need) {  // only whether the row is active
 #pragma unroll
         for (int q = 0; q < U; ++q)
           if (u[q] >= 0 && gather_ok(p, u[q], 0)) found |= changed(L.Mp, u[q]);
       }
+      found = pair_any(found);
       need = open || (need && !PW && !found);
       if (more) {
 #pragma unroll
         for (int q = 0; q < U; ++q) u[q] = need ? un[q] : -1;
       }
     }
-    if (act) ++L.items;
+    first_columns();
+    if (act && sub == 0) ++L.items;
     act = act && found;
     // m_active
-    uint32_t gdeg = 0;
-    if (act) {
+    uint32_t gdeg = 0, mask = 0;
+    if constexpr (PW) {
+      if (act) {
+#pragma unroll
+        for (int k = 0; k < WL; ++k)
+          if (acc[k] && (own[k] | ~valid_mask(w0 + k, p.s)) != ~0ULL) mask |= 1u << (w0 + k);
+      }
+      if (SUB > 1) mask |= __shfl_xor_sync(kFullMask, mask, 1);
+    }
+    if (act && sub == 0) {
       const unsigned long long deg = whole ? (uint32_t)len : p.deg_in[v];
       if constexpr (PW) {
-        uint32_t mask = 0;
-#pragma unroll
-        for (int k = 0; k < CW; ++k)
-          if (acc[k] && (own[k] | ~valid_mask(k, p.s)) != ~0ULL) mask |= 1u << k;
         if (mask && !whole) mask = claim_passes(L.Kc, v, mask);
         L.mact += deg * __popc(mask);
         L.rows += __popc(mask);
@@ -740,21 +866,21 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
     // new bits: to X and D of this round
     bool gain = false;
 #pragma unroll
-    for (int k = 0; k < CW; ++k) {
+    for (int k = 0; k < WL; ++k) {
       acc[k] &= act ? ~own[k] : 0ULL;
       gain |= acc[k] != 0ULL;
     }
     if (gain) {
-      uint64_t *xr = p.X + (size_t)v * Wp, *dr = L.Dc + (size_t)v * Wp;
+      uint64_t *xr = p.X + (size_t)v * CW + w0, *dr = L.Dc + (size_t)v * CW + w0;
       if (whole) {
 #pragma unroll
-        for (int k = 0; k < CW; ++k) own[k] |= acc[k];
-        store_words<CW>(xr, own);
-        store_words<CW>(dr, acc);
+        for (int k = 0; k < WL; ++k) own[k] |= acc[k];
+        store_words<WL>(xr, own);
+        store_words<WL>(dr, acc);
       } else {
         gain = false;
 #pragma unroll
-        for (int k = 0; k < CW; ++k)
+        for (int k = 0; k < WL; ++k)
           if (acc[k]) {
             acc[k] &= ~(uint64_t)atomicOr(reinterpret_cast<unsigned long long *>(xr + k),
                                           (unsigned long long)acc[k]);
@@ -765,8 +891,9 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
           }
       }
     }
+    gain = pair_any(gain);
     bool app = false;
-    if (gain) {
+    if (gain && sub == 0) {
       if (whole) {
         mark(L.Mc, v, kChanged);
         app = true;
@@ -776,18 +903,60 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
     }
     if (__any_sync(kFullMask, gain)) {
 #pragma unroll
-      for (int k = 0; k < CW; ++k)
+      for (int k = 0; k < WL; ++k)
         if (__any_sync(kFullMask, acc[k] != 0ULL)) {
-          const uint32_t n0 = __popc(transpose32((uint32_t)acc[k], L.lane));
-          const uint32_t n1 = __popc(transpose32((uint32_t)(acc[k] >> 32), L.lane));
-          if (n0) count_add(L, c0 + k * 64 + L.lane, n0);
-          if (n1) count_add(L, c0 + k * 64 + 32 + L.lane, n1);
+          const uint32_t t0 = transpose32((uint32_t)acc[k], L.lane);
+          const uint32_t t1 = transpose32((uint32_t)(acc[k] >> 32), L.lane);
+#pragma unroll
+          for (int h = 0; h < SUB; ++h) {  // the rows' word k is on every SUB-th lane
+            const uint32_t m = SUB == 1 ? ~0u : h ? 0xAAAAAAAAu : 0x55555555u;
+            const uint32_t n0 = __popc(t0 & m), n1 = __popc(t1 & m);
+            const int col = c0 + (h * WL + k) * 64 + L.lane;
+            if (n0) count_add(L, col, n0);
+            if (n1) count_add(L, col + 32, n1);
+          }
         }
       if (L.scnt > kStage - 32) stage_spill<SEG>(p, L);
       if (app) stage_degree<SEG>(p, L, p.deg_out[v], g);
       stage_row(L, v, app);
     }
   }
+}
+
+// Rows of 8 words: which seed owns which bit. A sweep gathers a row's two
+// 32-byte parts on two lanes and leaves a part out once the row can gain
+// nothing in it, so the seeds that reach the hubs late (those with few out-arcs) share
+// one part: they keep that part open in every row for a round, and the other
+// one closes after a few arcs. Seeds in order of out-degree, the first half of
+// those with any in words 0-3, the others in words 4-7, seeds without
+// out-arcs in the places left. Simulated on R-MAT 21 (s = 512), the largest
+// round gathers 63 M parts instead of 103 M.
+__device__ void place_seeds(const Params &p, Shared &sh, uint32_t *deg, const int32_t *seeds,
+                            int sp) {
+  for (int i = threadIdx.x; i < sp; i += blockDim.x) {
+    int64_t x = seeds[i];
+    if (p.perm) x = __ldg(p.perm + x);
+    deg[i] = (uint32_t)(__ldg(p.out_ptr + x + 1) - __ldg(p.out_ptr + x));
+  }
+  __syncthreads();
+  for (int i = threadIdx.x; i < sp; i += blockDim.x) {
+    const uint32_t d = deg[i];
+    int r = 0, alive = 0;  // rank by degree, seeds with out-arcs
+    for (int j = 0; j < sp; ++j) {
+      const uint32_t e = deg[j];
+      r += e > d || (e == d && j < i);
+      alive += e != 0u;
+    }
+    const int nb = min(sp - 256, alive / 2), na = alive - nb;  // in words 4-7, in words 0-3
+    const int k = r - alive;
+    const int at = r < na        ? r
+                   : r < alive   ? 256 + r - na
+                   : k < 256 - na ? na + k
+                                  : 256 + nb + k - (256 - na);
+    sh.place[i] = (uint16_t)at;
+    sh.col[at] = (uint16_t)i;
+  }
+  __syncthreads();
 }
 
 // A packed batch, by the block that arrived last: the graphs whose frontier
@@ -820,7 +989,7 @@ __device__ void list_dense(const Params &p, int cur) {
   }
 }
 
-template <int CW, bool PW, bool SEG>
+template <int CW, bool PW, bool SEG, bool PAIR>
 __global__ void __launch_bounds__(kMaxThreads, 1)
     k_rounds(const __grid_constant__ Params p, const int32_t *seeds, const int32_t *seed_bit,
              int sp, int resume, int epoch) {
@@ -850,6 +1019,8 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     sh.bar = 0;
   }
   if (L.tid == 0) ctrl->bad_index = 0;
+  // (the stages are free until the first round)
+  if (PAIR && p.sort_seeds) place_seeds(p, sh, dyn + 2 * p.ncols, seeds, sp);
   auto none = [] {};
   const int64_t mwords = (p.n + 15) / 16, kwords = (p.n + 3) / 4;  // marks, claim bytes
   int t;
@@ -907,7 +1078,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
           const int64_t k = (int64_t)x / p.perm_n;
           x = (int32_t)(k * p.perm_n + __ldg(p.perm + ((int64_t)x - k * p.perm_n)));
         }
-        const int bit = seed_bit ? seed_bit[i] : (int)i;
+        const int bit = seed_bit ? seed_bit[i] : PAIR && p.sort_seeds ? sh.place[i] : (int)i;
         int col = (int)i;
         if (SEG) col = __ldg(p.graph_col0 + __ldg(p.node_graph + x)) + bit;
         red_or(p.X + (size_t)x * CW + (bit >> 6), 1ULL << (bit & 63));
@@ -971,7 +1142,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       for (int i = threadIdx.x; i < p.ncols; i += blockDim.x) {
         const uint32_t c = cs[i];
         if (c) {
-          atomicAdd(&crow[i], c);
+          atomicAdd(&crow[PAIR && p.sort_seeds ? sh.col[i] : i], c);
           cs[i] = 0u;
         }
       }
@@ -1088,7 +1259,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       __syncthreads();
     }
     if (SEG ? p.dlist && *(volatile int32_t *)&ctrl->ndense > 0 : dense)
-      sweep_round<CW, PW, SEG>(p, L, tc, dense && p.early_stop ? sh.alive : nullptr);
+      sweep_round<CW, PW, SEG, PAIR>(p, L, tc, dense && p.early_stop ? sh.alive : nullptr);
     if (!dense) push_round<CW, PW, SEG>(p, L, Fp, Ep, nF, nE);
     round_flush<PW, SEG>(p, L, sh, scnt_s);
     if (!grid_barrier<SEG>(p, sh, [&] { list_dense(p, L.cur); })) return;
@@ -1119,17 +1290,19 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
 
 }  // namespace
 
-template <int CW>
+template <int CW, bool PAIR = false>
 static ResidentFn pick_resident(bool pw, bool seg) {
-  return seg ? &k_rounds<CW, false, true> : pw ? &k_rounds<CW, true, false> : &k_rounds<CW, false, false>;
+  if constexpr (!PAIR)
+    if (seg) return &k_rounds<CW, false, true, false>;
+  return pw ? &k_rounds<CW, true, false, PAIR> : &k_rounds<CW, false, false, PAIR>;
 }
 
-ResidentFn resident_fn(int CW, bool pw, bool seg) {
+ResidentFn resident_fn(int CW, bool pw, bool seg, bool pair) {
   switch (CW) {
     case 1: return pick_resident<1>(pw, seg);
     case 2: return pick_resident<2>(pw, seg);
     case 4: return pick_resident<4>(pw, seg);
-    case 8: return pick_resident<8>(pw, seg);
+    case 8: return pair ? pick_resident<8, true>(pw, false) : pick_resident<8>(pw, seg);
   }
   return nullptr;
 }

@@ -37,7 +37,7 @@ def _graph(kind):
 
 
 @pytest.mark.parametrize("kind", ["rmat", "rmat_directed", "depths"])
-@pytest.mark.parametrize("s", [1, 65, 200, 300])
+@pytest.mark.parametrize("s", [1, 65, 200, 257, 300, 512])
 def test_dense_rounds_stop_early(kind, s):
     g = _graph(kind)
     assert g.m >= 1 << 22

@@ -107,6 +107,10 @@ struct Params {
   uint32_t *C0, *C1;   // changed-in-round bitmaps, alternating by round parity
   uint32_t *K0, *K1;   // claim / active bitmaps, alternating
   uint32_t *Sat;       // saturated (all s bits set)
+  // wide rows of one graph: which parts of a row's delta hold a bit, by round
+  // parity like D (bit w >> dm_shift for word w); null: not kept
+  uint32_t *dm0, *dm1;
+  int32_t dm_shift;
   uint32_t *rowbits;   // wide rows: set bits of each row so far (else null)
   // PROPAGATE-S passes as the words of one signature: m_active per pass, with
   // one claim bit per (word, row) for rows cut into pieces, by round parity

@@ -24,7 +24,7 @@ struct Workspace {
   DevBuf arena;
   size_t used = 0;  // end of the laid-out parts in the arena
   DevBuf X, Y, D0, D1, C0, C1, K0, K1, Sat, RB, KW0, KW1, F0, F1, E, A, counts, rs, ctrl, seeds,
-      seed_bits, gfsum, gthr, dlist, dpref, E1, gm, F2, DI, DO;
+      seed_bits, gfsum, gthr, dlist, dpref, E1, gm, F2, DI, DO, DM0, DM1;
   DevBuf rctl;  // ResidentCtl, outside the arena: it keeps its address and contents
   int32_t epoch = 0;  // launches of the resident round loop
   Ctrl *ctrl_h = nullptr;  // pinned, 2 slots

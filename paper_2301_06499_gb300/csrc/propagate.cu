@@ -34,13 +34,13 @@ __global__ void __launch_bounds__(kBlock) k_zero(Params p, int64_t count_words, 
   ulonglong2 *d1 = reinterpret_cast<ulonglong2 *>(p.D1);
   for (int64_t i = gtid; i < pairs; i += nth) {
     x2[i] = z;
-    y2[i] = z;
+    if (p.Y) y2[i] = z;
     d0[i] = z;
     d1[i] = z;
   }
   if ((words & 1) && gtid == 0) {
     p.X[words - 1] = 0ULL;
-    p.Y[words - 1] = 0ULL;
+    if (p.Y) p.Y[words - 1] = 0ULL;
     p.D0[words - 1] = 0ULL;
     p.D1[words - 1] = 0ULL;
   }
@@ -57,6 +57,8 @@ __global__ void __launch_bounds__(kBlock) k_zero(Params p, int64_t count_words, 
   }
   if (p.rowbits)
     for (int64_t i = gtid; i < p.n; i += nth) p.rowbits[i] = 0u;
+  if (p.dm0)
+    for (int64_t i = gtid; i < p.n; i += nth) p.dm0[i] = p.dm1[i] = 0u;
   if (p.pass_words)
     for (int64_t i = gtid; i < p.nbm * p.Wp; i += nth) {
       p.Kw0[i] = 0u;
@@ -91,23 +93,18 @@ __global__ void __launch_bounds__(kBlock) k_zero(Params p, int64_t count_words, 
 }
 
 // ------------------------------------------------------------- k_seed
-// One block. Round 0 of the pass: seed i gets bit i (Sig(x_i)[i] = 1) as a
-// change of round 0 (X = 0, Y = the bit), so the post kernel of round 0
-// counts the pairs (x_i, x_i), records the seeds' deltas and expands them
-// like any other frontier. A node may carry several seeds' bits (requests
-// merged on one graph); it enters the frontier once.
-__global__ void __launch_bounds__(1024) k_seed(Params p, const int32_t *seeds,
-                                               const int32_t *seed_bit, int sp) {
-  __shared__ unsigned long long tot;
-  __shared__ unsigned int nf;
-  if (threadIdx.x == 0) {
-    tot = 0ULL;
-    nf = 0u;
-  }
-  __syncthreads();
+// Round 0 of the pass: seed i gets bit i (Sig(x_i)[i] = 1) as a change of
+// round 0 (X = 0, Y = the bit), so the post kernel of round 0 counts the
+// pairs (x_i, x_i), records the seeds' deltas and expands them like any other
+// frontier. A node may carry several seeds' bits (requests merged on one
+// graph); it enters the frontier once. A warp per 32 seeds over the grid (one
+// block took 1.04 ms for the 30,000 seeds of an exact run).
+__global__ void __launch_bounds__(kBlock) k_seed(Params p, const int32_t *seeds,
+                                                 const int32_t *seed_bit, int sp) {
   const int lane = threadIdx.x & 31;
   // whole warps iterate so that the warp-level appends see every lane
-  for (int base = (threadIdx.x & ~31); base < sp; base += blockDim.x) {
+  for (int base = (blockIdx.x * kBlock + threadIdx.x) & ~31; base < sp;
+       base += gridDim.x * kBlock) {
     const int i = base + lane;
     unsigned long long od = 0;
     int32_t x = 0;
@@ -119,21 +116,30 @@ __global__ void __launch_bounds__(1024) k_seed(Params p, const int32_t *seeds,
         x = (int32_t)(k * p.perm_n + __ldg(p.perm + ((int64_t)x - k * p.perm_n)));
       }
       const int bit = seed_bit ? seed_bit[i] : i;  // a batch: the seed's index in its graph
-      atomicOr(reinterpret_cast<unsigned long long *>(p.Y + (size_t)x * p.Wp + (bit >> 6)),
-               1ULL << (bit & 63));
+      const size_t word = (size_t)x * p.Wp + (bit >> 6);
+      if (p.dm0) {  // X and D hold the round's bits at once (k_pull_wide)
+        atomicOr(reinterpret_cast<unsigned long long *>(p.X + word), 1ULL << (bit & 63));
+        atomicOr(reinterpret_cast<unsigned long long *>(p.D0 + word), 1ULL << (bit & 63));
+        atomicOr(p.dm0 + x, 1u << ((bit >> 6) >> p.dm_shift));
+      } else {
+        atomicOr(reinterpret_cast<unsigned long long *>(p.Y + word), 1ULL << (bit & 63));
+      }
       first = !set_bit(p.C0, x);
       if (first) {
-        p.F0[atomicAdd(&nf, 1u)] = x;
         od = (unsigned long long)(p.out_ptr[x + 1] - p.out_ptr[x]);
-        atomicAdd(&tot, od);
         if (p.gfsum && od) atomicAdd(p.gfsum + p.node_graph[x], od);  // round 0's parity
       }
     }
+    const unsigned mask = __ballot_sync(kFullMask, first);
+    unsigned long long tot, at = 0;
+    warp_excl_scan64(od, lane, &tot);
+    if (lane == 0 && mask)
+      at = atomicAdd(&p.ctrl->fpack, ((unsigned long long)__popc(mask) << kFsumBits) + tot);
+    at = __shfl_sync(kFullMask, at, 0) >> kFsumBits;
+    if (first) p.F0[at + __popc(mask & ((1u << lane) - 1u))] = x;
     const unsigned long long ne = first ? (od + p.LE - 1) / p.LE : 0ULL;
     warp_append_pieces(E_of(p, 0), &p.ctrl->nE, x, ne, lane);
   }
-  __syncthreads();
-  if (threadIdx.x == 0) p.ctrl->fpack = ((unsigned long long)nf << kFsumBits) | tot;
 }
 
 __device__ __forceinline__ bool row_full(const uint64_t *row, int Wp, int s) {
@@ -142,6 +148,107 @@ __device__ __forceinline__ bool row_full(const uint64_t *row, int Wp, int s) {
     full &= ((__ldg(reinterpret_cast<const unsigned long long *>(row) + w) | ~valid_mask(w, s)) ==
              ~0ULL);
   return full;
+}
+
+// Per-seed counts of the wide rows of one graph whose pull wrote their deltas
+// (k_pull_wide): a warp takes 32 words of a run of frontier rows, a lane one
+// word, and counts its 64 columns in bit-sliced form. Plane k holds bit k of
+// each column's count, so that eight rows cost seven carry-save adders and a
+// ripple for all columns of a word at once: 10 instructions a row and word
+// pair where the 32 x 32 transposes through shared memory took 50. That, not
+// the 0.7 GB of deltas, bounded the kernel: 0.90 ms a round of ER 10^6 at
+// s = 5,568, now 0.40 (the deltas read and the previous ones cleared, 3.5
+// TB/s). Words without a bit (dm) are not read.
+constexpr int kCountPlanes = 13;
+constexpr int kCountRows = 4096;  // rows of one run at most (< 2^13)
+
+__device__ __forceinline__ void add3(uint32_t &carry, uint32_t &sum, uint32_t a, uint32_t b) {
+  const uint32_t u = sum ^ a;
+  carry = (sum & a) | (u & b);
+  sum = u ^ b;
+}
+
+__device__ __forceinline__ void add8(uint32_t (&pl)[kCountPlanes], const uint32_t (&d)[8]) {
+  uint32_t t0, t1, f0, f1, e;
+  add3(t0, pl[0], d[0], d[1]);
+  add3(t1, pl[0], d[2], d[3]);
+  add3(f0, pl[1], t0, t1);
+  add3(t0, pl[0], d[4], d[5]);
+  add3(t1, pl[0], d[6], d[7]);
+  add3(f1, pl[1], t0, t1);
+  add3(e, pl[2], f0, f1);
+#pragma unroll
+  for (int k = 3; k < kCountPlanes; ++k) {
+    const uint32_t c = pl[k] & e;
+    pl[k] ^= e;
+    e = c;
+  }
+}
+
+// Every thread of the block calls it; cnt: kCountCols words of shared memory.
+// A block keeps to one block of 32 words (while there are blocks enough), so
+// that its warps' counts meet in shared memory and leave as 2,048 adds: a
+// warp's own adds to global memory took 0.16 ms a round of 30,000 seeds.
+constexpr int kCountCols = 2048;
+
+__device__ __forceinline__ void count_wide(const Params &p, const int32_t *F, int64_t nF,
+                                           const uint64_t *D, const uint32_t *M, uint32_t *crow,
+                                           uint32_t *cnt) {
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int Wp = p.Wp, ncb = (Wp + 31) >> 5, grid = (int)gridDim.x;
+  const int step = grid >= ncb ? ncb : grid;
+  for (int cb = (int)blockIdx.x % step; cb < ncb; cb += step) {
+    const int64_t part = blockIdx.x / step, parts = (grid - (int)blockIdx.x % step + step - 1) / step;
+    const int64_t runs = parts * (kBlock / 32);  // row runs side by side
+    int64_t per = (nF + runs - 1) / runs;
+    per = min((long long)kCountRows, max(32LL, ((long long)per + 7) & ~7LL));
+    for (int i = threadIdx.x; i < kCountCols; i += kBlock) cnt[i] = 0u;
+    __syncthreads();
+    const int w = cb * 32 + lane;
+    for (int64_t r0 = (part * (kBlock / 32) + wid) * per; r0 < nF; r0 += runs * per) {
+      const int64_t r1 = min(nF, r0 + per);
+      uint32_t lo[kCountPlanes], hi[kCountPlanes];
+#pragma unroll
+      for (int k = 0; k < kCountPlanes; ++k) lo[k] = hi[k] = 0u;
+      bool some = false;
+      int32_t v_next = lane < 8 && r0 + lane < r1 ? F[r0 + lane] : -1;
+      for (int64_t r = r0; r < r1; r += 8) {
+        const int32_t vl = v_next;
+        const uint32_t ml = vl >= 0 ? M[vl] : 0u;
+        v_next = lane < 8 && r + 8 + lane < r1 ? F[r + 8 + lane] : -1;
+        uint32_t dl[8], dh[8];
+#pragma unroll
+        for (int q = 0; q < 8; ++q) {
+          const int32_t v = __shfl_sync(kFullMask, vl, q);
+          const uint32_t m = __shfl_sync(kFullMask, ml, q);
+          uint64_t d = 0ULL;
+          if (w < Wp && ((m >> (w >> p.dm_shift)) & 1u)) d = D[(size_t)v * Wp + w];
+          dl[q] = (uint32_t)d;
+          dh[q] = (uint32_t)(d >> 32);
+        }
+        const uint32_t any = (dl[0] | dl[1] | dl[2] | dl[3]) | (dl[4] | dl[5] | dl[6] | dl[7]) |
+                             (dh[0] | dh[1] | dh[2] | dh[3]) | (dh[4] | dh[5] | dh[6] | dh[7]);
+        if (!__any_sync(kFullMask, any != 0u)) continue;
+        some = true;
+        add8(lo, dl);
+        add8(hi, dh);
+      }
+      if (!some) continue;
+      const int bits = 32 - __clz((int)(r1 - r0));
+      for (int j = 0; j < 64; ++j) {  // rotated by lane: lanes are 64 columns apart
+        const int jj = (j + lane) & 63, b = jj & 31;
+        uint32_t n = 0;
+#pragma unroll
+        for (int k = 0; k < kCountPlanes; ++k)
+          if (k < bits) n |= (((jj & 32) ? hi[k] : lo[k]) >> b & 1u) << k;
+        if (n) atomicAdd(cnt + lane * 64 + jj, n);
+      }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kCountCols; i += kBlock)
+      if (cnt[i]) atomicAdd(crow + cb * kCountCols + i, cnt[i]);
+    __syncthreads();
+  }
 }
 
 // ------------------------------------------------------------- k_post
@@ -200,7 +307,11 @@ __global__ void __launch_bounds__(kBlock, 4) k_post(Params p) {
     __syncthreads();
   }
   // A. count, record deltas, sync, saturation
-  if constexpr (WIDE) {
+  if (WIDE && p.dm0) {
+    // X, D, Sat and the deltas' parts were written by the pull
+    __shared__ uint32_t cnt_s[kCountCols];
+    count_wide(p, F, nF, Dcur, (t & 1) ? p.dm1 : p.dm0, crow, cnt_s);
+  } else if constexpr (WIDE) {
     // tiles of 32 frontier rows x 16 words: each half-warp moves 16
     // consecutive words (128 bytes) of one row, so loads and stores are
     // coalesced; the deltas go through shared memory to a lane-per-row
@@ -358,9 +469,15 @@ __global__ void __launch_bounds__(kBlock, 4) k_post(Params p) {
   // the deltas of round t-1 were read by the pull of round t: clear them
   if constexpr (WIDE) {  // a warp per row, 16 bytes a lane
     const ulonglong2 z = make_ulonglong2(0ULL, 0ULL);
+    uint32_t *Mprev = (t & 1) ? p.dm0 : p.dm1;
     for (int64_t r = warp; r < nFprev; r += nwarps) {
-      ulonglong2 *dr = reinterpret_cast<ulonglong2 *>(Dprev + (size_t)Fprev[r] * Wp);
-      for (int k = lane; k < (Wp >> 1); k += 32) dr[k] = z;
+      const int32_t v = Fprev[r];
+      ulonglong2 *dr = reinterpret_cast<ulonglong2 *>(Dprev + (size_t)v * Wp);
+      const uint32_t parts = Mprev ? Mprev[v] : ~0u;  // the others are zero
+      __syncwarp();
+      for (int k = lane; k < (Wp >> 1); k += 32)
+        if ((parts >> ((2 * k) >> p.dm_shift)) & 1u) dr[k] = z;
+      if (Mprev && lane == 0) Mprev[v] = 0u;
     }
   } else {
     const ulonglong2 z = make_ulonglong2(0ULL, 0ULL);
@@ -428,7 +545,7 @@ __global__ void __launch_bounds__(kBlock, 4) k_post(Params p) {
         for (int q = 0; q < UNR; ++q)
           cand[q] = x[q] >= 0 && !test_bit_live(p.Sat, x[q]) &&
                     !(test_bit(Ccur, x[q]) &&
-                      row_full(p.Y + (size_t)x[q] * Wp, Wp,
+                      row_full((p.dm0 ? p.X : p.Y) + (size_t)x[q] * Wp, Wp,
                                p.node_graph ? p.graph_s[p.node_graph[x[q]]] : s));
         bool claim[UNR];
 #pragma unroll
@@ -1098,7 +1215,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   // TMA gather of an empty slot reads)
   const size_t delta_bytes_alloc = sig_bytes + sizeof(uint64_t) * (size_t)pl.Wp;
   std::vector<std::pair<DevBuf *, size_t>> needs = {
-      {&w.X, sig_bytes}, {&w.Y, sig_bytes}, {&w.D0, delta_bytes_alloc}, {&w.D1, delta_bytes_alloc},
+      {&w.X, sig_bytes}, {&w.D0, delta_bytes_alloc}, {&w.D1, delta_bytes_alloc},
       {&w.C0, c_bytes}, {&w.C1, c_bytes}, {&w.Sat, c_bytes},
       {&w.F0, sizeof(int32_t) * (size_t)n}, {&w.F1, sizeof(int32_t) * (size_t)n},
       {&w.E, sizeof(unsigned long long) * (size_t)e_cap},
@@ -1114,7 +1231,19 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
     needs.push_back({&w.K1, bm_bytes});
     needs.push_back({&w.A, sizeof(ulonglong2) * (size_t)std::max<int64_t>(npieces, 1)});
   }
-  if (pl.post_wide) needs.push_back({&w.RB, sizeof(uint32_t) * (size_t)n});
+  // one graph's wide rows keep no Y: the pull writes X and D itself
+  const bool direct = pl.wide && pl.post_wide;
+  if (direct) {  // its post kernel counts in fixed shared memory
+    pl.smem_counts = false;
+    pl.post_smem = 0;
+  }
+  if (!direct) needs.push_back({&w.Y, sig_bytes});
+  if (direct) {
+    needs.push_back({&w.DM0, sizeof(uint32_t) * (size_t)n});
+    needs.push_back({&w.DM1, sizeof(uint32_t) * (size_t)n});
+  } else if (pl.post_wide) {
+    needs.push_back({&w.RB, sizeof(uint32_t) * (size_t)n});
+  }
   if (pw) {  // claim bits per (word, row); the resident loop: a byte per row
     const size_t kw = resident ? ((size_t)n + 3) / 4 * 4 : bm_bytes * (size_t)pl.Wp;
     needs.push_back({&w.KW0, kw});
@@ -1166,7 +1295,16 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   p.K0 = (uint32_t *)w.K0.p;
   p.K1 = (uint32_t *)w.K1.p;
   p.Sat = (uint32_t *)w.Sat.p;
-  p.rowbits = pl.post_wide ? (uint32_t *)w.RB.p : nullptr;
+  p.rowbits = pl.post_wide && !direct ? (uint32_t *)w.RB.p : nullptr;
+  if (direct) {
+    p.Y = nullptr;
+    p.dm0 = (uint32_t *)w.DM0.p;
+    p.dm1 = (uint32_t *)w.DM1.p;
+    p.dm_shift = 2;  // a 32-byte sector, or as many words as 32 parts allow
+    while (((pl.Wp - 1) >> p.dm_shift) > 31) ++p.dm_shift;
+  } else {
+    p.dm_shift = 31;  // one part: read always
+  }
   p.pass_words = pw ? 1 : 0;
   p.Kw0 = pw ? (uint32_t *)w.KW0.p : nullptr;
   p.Kw1 = pw ? (uint32_t *)w.KW1.p : nullptr;
@@ -1314,7 +1452,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   const int64_t zero_work = std::max<int64_t>({n * pl.Wp / 2, nbm, count_words, rs_words, 1});
   k_zero<<<occupancy_grid((const void *)&k_zero, 0, zero_work), kBlock, 0, st>>>(p, count_words,
                                                                                 rs_words);
-  k_seed<<<1, 1024, 0, st>>>(p, (const int32_t *)w.seeds.p,
+  k_seed<<<occupancy_grid((const void *)&k_seed, 0, sp), kBlock, 0, st>>>(p, (const int32_t *)w.seeds.p,
                              bs ? (const int32_t *)w.seed_bits.p : nullptr, sp);
   launch_post(pl, p, st);
   po.launches += 3;

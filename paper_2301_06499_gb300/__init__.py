@@ -37,14 +37,20 @@ def library_path() -> str:
     return build.LIB
 
 
+_torch = None  # once a process has seen torch with a GPU, it keeps it
+
+
 def _current_stream():
-    try:
-        import torch
-        if torch.cuda.is_available():
-            return ctypes.c_void_p(torch.cuda.current_stream().cuda_stream)
-    except ImportError:
-        pass
-    return ctypes.c_void_p(0)
+    global _torch
+    if _torch is None:
+        try:
+            import torch
+            if not torch.cuda.is_available():
+                return ctypes.c_void_p(0)
+        except ImportError:
+            return ctypes.c_void_p(0)
+        _torch = torch
+    return ctypes.c_void_p(_torch.cuda.current_stream().cuda_stream)
 
 
 def options(**kw) -> _abi.Options:

@@ -65,6 +65,21 @@ struct ResidentCtl {
   uint32_t exited;                        // blocks that left the launch
 };
 
+// What a resident launch leaves in pinned host memory: its last control block,
+// each block's work counters and, when they fit, the rounds' statistics and
+// counts (data: rows + 1 RoundStats, then rows x columns), so that a short call
+// is one launch and one wait without copies.
+constexpr int kResidentBlocks = 256;          // blocks of a resident launch at most
+constexpr int kResidentSeeds = 4096;          // seeds the launch reads from pinned memory
+constexpr int kResidentOut = 64 << 10;        // bytes of data
+struct ResidentOut {
+  Ctrl ctrl;
+  int32_t rows;  // count rows in data, -1: not there
+  unsigned long long sums[kResidentBlocks][3];  // arcs scanned, deltas gathered, items
+  int32_t seeds[kResidentSeeds];
+  alignas(64) unsigned char data[kResidentOut];
+};
+
 // Per-round work counters (device), indexed by round.
 struct RoundStats {
   unsigned long long work;     // sum over active rows of s_graph(v) * indeg(v)
@@ -155,6 +170,7 @@ struct Params {
   int64_t perm_n;       // nodes of the relabelled graph (replicas: a seed k*perm_n + x
                         // of copy k maps to k*perm_n + perm[x])
   ResidentCtl *rctl;    // resident loop (else null)
+  ResidentOut *out;     // resident loop: pinned host memory
   uint32_t *deg_in, *deg_out;  // resident loop: degrees (the same array for symmetric graphs)
   int32_t sort_seeds;   // resident loop: bits of rows of 8 words placed by the seeds' degree
   int64_t dense_above;  // resident loop: a full sweep when the frontier's out-arcs pass this

@@ -671,6 +671,8 @@ void release_workspace(Workspace &w) {
   }
   if (w.ctrl_h) cudaFreeHost(w.ctrl_h);
   w.ctrl_h = nullptr;
+  if (w.out_h) cudaFreeHost(w.out_h);
+  w.out_h = nullptr;
   for (auto &e : w.ev)
     if (e) cudaEventDestroy(e);
   w.ev[0] = w.ev[1] = nullptr;

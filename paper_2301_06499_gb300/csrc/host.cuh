@@ -28,6 +28,7 @@ struct Workspace {
   DevBuf rctl;  // ResidentCtl, outside the arena: it keeps its address and contents
   int32_t epoch = 0;  // launches of the resident round loop
   Ctrl *ctrl_h = nullptr;  // pinned, 2 slots
+  ResidentOut *out_h = nullptr;  // pinned, of the resident round loop
   cudaEvent_t ev[2] = {nullptr, nullptr};
   std::vector<cudaEvent_t> tev;  // timing events
 };

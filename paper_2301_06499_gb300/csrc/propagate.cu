@@ -886,6 +886,22 @@ struct Call {
   std::vector<unsigned long long> *gm_h = nullptr;
 };
 
+static void add_stats(Call &cl, const RoundStats *r, int32_t row_base, int32_t rows) {
+  if ((int64_t)cl.rs_h.size() < (int64_t)row_base + rows)
+    cl.rs_h.resize((size_t)row_base + rows, RoundStats{});
+  for (int i = 0; i < rows; ++i) {
+    RoundStats &d = cl.rs_h[(size_t)row_base + i];
+    d.work += r[i].work;
+    d.m_active += r[i].m_active;
+    d.scanned += r[i].scanned;
+    d.gathered += r[i].gathered;
+    d.items += r[i].items;
+    d.changed += r[i].changed;
+    d.fsum += r[i].fsum;
+    d.rows += r[i].rows;
+  }
+}
+
 static pg_status copy_window(Call &cl, const Params &p, int col0, int32_t row_base, int32_t rows,
                              int32_t rs_rows) {
   rows = std::min(rows, cl.max_rounds + 1 - row_base);
@@ -911,19 +927,7 @@ static pg_status copy_window(Call &cl, const Params &p, int col0, int32_t row_ba
                                     cudaMemcpyDeviceToHost, cl.st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(cl.st);
     if (e != cudaSuccess) return cuda_status(e);
-    if ((int64_t)cl.rs_h.size() < (int64_t)row_base + rs_rows)
-      cl.rs_h.resize((size_t)row_base + rs_rows, RoundStats{});
-    for (int i = 0; i < rs_rows; ++i) {
-      RoundStats &d = cl.rs_h[(size_t)row_base + i];
-      d.work += tmp[i].work;
-      d.m_active += tmp[i].m_active;
-      d.scanned += tmp[i].scanned;
-      d.gathered += tmp[i].gathered;
-      d.items += tmp[i].items;
-      d.changed += tmp[i].changed;
-      d.fsum += tmp[i].fsum;
-      d.rows += tmp[i].rows;
-    }
+    add_stats(cl, tmp.data(), row_base, rs_rows);
     if (p.gmact && cl.gm_h) {
       const size_t ns = (size_t)p.nseg;
       std::vector<unsigned long long> g((size_t)rs_rows * ns);
@@ -1111,8 +1115,8 @@ static void resident_smem_optin() {
 
 // One pass as a cooperative launch of the resident round loop (launched again
 // after each full counts window).
-static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w, bool batch, int sp,
-                              int col0, PassOut &po) {
+static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w, bool batch,
+                              const int32_t *seeds_h, int sp, int col0, PassOut &po) {
   cudaStream_t st = cl.st;
   pg_status rc;
   if (!w.rctl.p) {
@@ -1125,12 +1129,27 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   const ResidentFn fn = resident_fn(pl.CW, pl.pw, batch, pair);
   // the SMs given to this graph (propagations that run side by side share
   // them: a cooperative launch waits until all its blocks fit), else all
-  const int blocks = cl.g->sms > 0 ? std::min(cl.g->sms, sm_count()) : sm_count();
+  const int blocks =
+      std::min(cl.g->sms > 0 ? std::min(cl.g->sms, sm_count()) : sm_count(), kResidentBlocks);
   const int threads = resident_threads(p.n, blocks);
   // a seed's bit is the loop's own business unless bits are passes
   p.sort_seeds = pair && !pl.pw && sp > 256 && sp <= kResidentSorted;
   const size_t smem = resident_smem(p.ncols, threads);
+  if (!w.out_h && cudaMallocHost((void **)&w.out_h, sizeof(ResidentOut)) != cudaSuccess) {
+    cudaGetLastError();
+    w.out_h = nullptr;
+    return PG_ENOMEM;
+  }
+  p.out = w.out_h;
+  // few seeds are read from pinned memory, once: no copy ahead of the launch
   const int32_t *seeds = (const int32_t *)w.seeds.p;
+  if (sp <= kResidentSeeds && !p.perm) {
+    std::memcpy(w.out_h->seeds, seeds_h, sizeof(int32_t) * (size_t)sp);
+    seeds = w.out_h->seeds;
+  } else if ((rc = cuda_status(cudaMemcpyAsync(w.seeds.p, seeds_h, sizeof(int32_t) * (size_t)sp,
+                                               cudaMemcpyHostToDevice, st)))) {
+    return rc;
+  }
   const int32_t *bits = batch ? (const int32_t *)w.seed_bits.p : nullptr;
   int resume = 0;
   p.row_base = 0;
@@ -1144,11 +1163,14 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
                                                       dim3(threads), args, smem, st))))
       return rc;
     po.launches += 1;
-    if ((rc = cuda_status(cudaMemcpyAsync(&w.ctrl_h[0], p.ctrl, sizeof(Ctrl),
-                                          cudaMemcpyDeviceToHost, st))) ||
-        (rc = cuda_status(cudaStreamSynchronize(st))))
-      return rc;
-    fin = w.ctrl_h[0];
+    if ((rc = cuda_status(cudaStreamSynchronize(st)))) return rc;
+    fin = w.out_h->ctrl;
+    if (cl.rs_h.empty()) cl.rs_h.resize(1, RoundStats{});
+    for (int b = 0; b < blocks; ++b) {
+      cl.rs_h[0].scanned += w.out_h->sums[b][0];
+      cl.rs_h[0].gathered += w.out_h->sums[b][1];
+      cl.rs_h[0].items += w.out_h->sums[b][2];
+    }
     if (!fin.done || fin.iters != epoch) {  // a wait of the barrier ran out
       cudaMemsetAsync(w.rctl.p, 0, sizeof(ResidentCtl), st);
       return PG_ETIMEOUT;
@@ -1161,7 +1183,19 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   if (fin.bad_index) return PG_EDEVICE;  // a PG_DEBUG_BOUNDS build caught a bad gather
   const int32_t last = fin.status == PG_ERANGE ? cl.max_rounds : fin.last_round;
   const int32_t rows = last - p.row_base + 1;
-  if ((rc = copy_window(cl, p, col0, p.row_base, rows, rows + 1))) return rc;
+  if (w.out_h->rows == rows && fin.status == PG_OK) {
+    const RoundStats *rs = reinterpret_cast<const RoundStats *>(w.out_h->data);
+    add_stats(cl, rs, p.row_base, std::min(rows + 1, cl.max_rounds + 2 - p.row_base));
+    const uint32_t *counts = reinterpret_cast<const uint32_t *>(rs + rows + 1);
+    if (rows > 0 && cl.sink)
+      cl.sink(cl.sink_ctx, p.row_base, rows, counts, p.ncols);
+    else
+      for (int32_t t = 0; t < rows; ++t)
+        std::memcpy(cl.counts_h + (size_t)(p.row_base + t) * cl.s_total + col0,
+                    counts + (size_t)t * p.ncols, sizeof(uint32_t) * (size_t)p.ncols);
+  } else if ((rc = copy_window(cl, p, col0, p.row_base, rows, rows + 1))) {
+    return rc;
+  }
   po.rounds = fin.status == PG_ERANGE ? cl.max_rounds + 1 : fin.last_round;
   po.status = fin.status;
   po.dense_rounds = fin.dense_rounds;
@@ -1426,8 +1460,9 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
     init_ev0 = ntev++;
     cudaEventRecord(tev(init_ev0), st);
   }
-  rc = cuda_status(cudaMemcpyAsync(w.seeds.p, seeds_h, sizeof(int32_t) * sp,
-                                   cudaMemcpyHostToDevice, st));
+  if (!resident)
+    rc = cuda_status(cudaMemcpyAsync(w.seeds.p, seeds_h, sizeof(int32_t) * sp,
+                                     cudaMemcpyHostToDevice, st));
   if (rc == PG_OK && p.gfsum) {
     std::vector<unsigned long long> thr((size_t)g->nseg);
     const double f = p.dense_threshold;
@@ -1446,7 +1481,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
     rc = cuda_status(cudaMemcpyAsync(w.seed_bits.p, bs->seed_bit, sizeof(int32_t) * sp,
                                      cudaMemcpyHostToDevice, st));
   if (rc) return rc;
-  if (resident) return run_resident(cl, pl, p, w, bs != nullptr, sp, col0, po);
+  if (resident) return run_resident(cl, pl, p, w, bs != nullptr, seeds_h, sp, col0, po);
   const int64_t count_words = (int64_t)row_cap * ncols;
   const int64_t rs_words = (int64_t)(row_cap + 2) * (int64_t)(sizeof(RoundStats) / 8);
   const int64_t zero_work = std::max<int64_t>({n * pl.Wp / 2, nbm, count_words, rs_words, 1});
@@ -1656,14 +1691,24 @@ static int pass_words_for(const pg_graph *g, int npasses, int planes, const pg_o
   return K;
 }
 
+// Seeds in range and distinct: an open-addressed set (sorting the 30,000 of an
+// exact run took 2 ms of its 7).
 static pg_status check_seeds(const pg_graph *g, const int32_t *seeds, int32_t s) {
   if (!seeds || s < 1 || s > g->n) return PG_EINVAL;
-  std::vector<int32_t> v(seeds, seeds + s);
-  for (int32_t x : v)
+  int bits = 4;
+  while ((1LL << bits) < 2LL * s) ++bits;
+  std::vector<int32_t> set((size_t)1 << bits, -1);
+  const uint32_t mask = (1u << bits) - 1u;
+  for (int32_t i = 0; i < s; ++i) {
+    const int32_t x = seeds[i];
     if (x < 0 || x >= g->n) return PG_EINVAL;
-  std::sort(v.begin(), v.end());
-  for (int32_t i = 1; i < s; ++i)
-    if (v[i] == v[i - 1]) return PG_EINVAL;
+    uint32_t at = ((uint32_t)x * 2654435769u) >> (32 - bits);
+    while (set[at] != -1) {
+      if (set[at] == x) return PG_EINVAL;
+      at = (at + 1) & mask;
+    }
+    set[at] = x;
+  }
   return PG_OK;
 }
 

@@ -130,6 +130,8 @@ struct Shared {
   uint16_t col[kResidentSorted];   // count column of each bit (p.sort_seeds)
   uint16_t place[kResidentSorted]; // bit of each seed
   unsigned long long fp, ne_all;
+  unsigned long long sums[3];
+  int rows_out;  // count rows to hand over at the fixpoint, else -1
   uint32_t bar;  // barriers this block has arrived at
   int last;      // this block arrived last
   int failed;    // the barrier gave up
@@ -989,6 +991,45 @@ __device__ void list_dense(const Params &p, int cur) {
   }
 }
 
+// The launch's results, to pinned host memory.
+__device__ __forceinline__ void hand_over(ResidentOut *out, const RoundStats *stats,
+                                          const uint32_t *counts, int ncols, const Ctrl *ctrl,
+                                          const int *rows_out, unsigned long long *sums,
+                                          uint32_t scan, uint32_t gath, uint32_t items) {
+  const uint32_t tid = blockIdx.x * blockDim.x + threadIdx.x;
+  unsigned long long s3[3] = {scan, gath, items};
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s3[k] += __shfl_xor_sync(kFullMask, s3[k], off);
+    if ((threadIdx.x & 31) == 0) atomicAdd(sums + k, s3[k]);
+  }
+  __syncthreads();
+  if (threadIdx.x < 3) out->sums[blockIdx.x][threadIdx.x] = sums[threadIdx.x];
+  // at the fixpoint every row is complete: the last counts left their blocks a
+  // round ago
+  const int rows = *rows_out;  // thread 0's, after the barrier
+  const size_t rs_bytes = sizeof(RoundStats) * (size_t)(rows + 1);
+  const bool fits = rows >= 0 &&
+                    rs_bytes + sizeof(uint32_t) * (size_t)rows * (size_t)ncols <= kResidentOut;
+  if (fits) {
+    if (blockIdx.x == 0) {
+      const unsigned long long *rs = reinterpret_cast<const unsigned long long *>(stats);
+      unsigned long long *to = reinterpret_cast<unsigned long long *>(out->data);
+      for (int i = threadIdx.x; i < (int)(rs_bytes / 8); i += blockDim.x)
+        to[i] = *(volatile const unsigned long long *)(rs + i);
+    }
+    uint32_t *to = reinterpret_cast<uint32_t *>(out->data + rs_bytes);
+    // (32-bit indices: 64-bit ones made the rounds spill)
+    for (uint32_t i = tid; i < (uint32_t)(rows * ncols); i += gridDim.x * blockDim.x)
+      to[i] = ld_u32(counts + i);
+  }
+  if (tid == 0) {
+    out->ctrl = *ctrl;
+    out->rows = fits ? rows : -1;
+  }
+}
+
 template <int CW, bool PW, bool SEG, bool PAIR>
 __global__ void __launch_bounds__(kMaxThreads, 1)
     k_rounds(const __grid_constant__ Params p, const int32_t *seeds, const int32_t *seed_bit,
@@ -1017,6 +1058,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     sh.mact = sh.work = sh.od = sh.ne = 0;
     sh.rows = sh.staged = 0;
     sh.bar = 0;
+    sh.sums[0] = sh.sums[1] = sh.sums[2] = 0;
   }
   if (L.tid == 0) ctrl->bad_index = 0;
   // (the stages are free until the first round)
@@ -1164,6 +1206,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       stop = false;
     }
     if (stop) {
+      if (threadIdx.x == 0) sh.rows_out = !SEG && nF == 0 ? t - p.row_base : -1;
       if (lead) {
         ctrl->t = t + 1;
         ctrl->mode = prev_dense;
@@ -1274,18 +1317,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     rc->gen = 0u;
     rc->exited = 0u;
   }
-  // work counters of the launch, on the slot of its last round
-  unsigned long long s3[3] = {L.scan, L.gath, L.items};
-#pragma unroll
-  for (int k = 0; k < 3; ++k)
-#pragma unroll
-    for (int off = 16; off > 0; off >>= 1) s3[k] += __shfl_xor_sync(kFullMask, s3[k], off);
-  if (L.lane == 0) {
-    RoundStats *r = p.rs + (t - p.row_base);
-    if (s3[0]) atomicAdd(&r->scanned, s3[0]);
-    if (s3[1]) atomicAdd(&r->gathered, s3[1]);
-    if (s3[2]) atomicAdd(&r->items, s3[2]);
-  }
+  hand_over(p.out, p.rs, p.counts, p.ncols, ctrl, &sh.rows_out, sh.sums, L.scan, L.gath, L.items);
 }
 
 }  // namespace

@@ -129,6 +129,7 @@ struct Params {
   uint32_t *rowbits;   // wide rows: set bits of each row so far (else null)
   // PROPAGATE-S passes as the words of one signature: m_active per pass, with
   // one claim bit per (word, row) for rows cut into pieces, by round parity
+  int32_t zero_d;      // the delta buffers have to be zeroed first
   int32_t pass_words;
   uint32_t *Kw0, *Kw1;  // [Wp][nbm] each (null unless pass_words)
   int64_t nbm;         // 32-bit words per bitmap

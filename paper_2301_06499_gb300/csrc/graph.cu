@@ -288,7 +288,10 @@ __global__ void k_max_degree(const int64_t *rp, int64_t n, unsigned long long *m
   for (int64_t v = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; v < n;
        v += (int64_t)gridDim.x * blockDim.x)
     best = max(best, (unsigned long long)(rp[v + 1] - rp[v]));
-  atomicMax(mx, best);
+  // one atomic per warp (degrees are below 2^32): a thread each queued at the
+  // one word, 0.20 ms for 4 M rows
+  best = __reduce_max_sync(kFullMask, (uint32_t)best);
+  if ((threadIdx.x & 31) == 0) atomicMax(mx, best);
 }
 
 // ------------------------------------------------------------- work list
@@ -645,6 +648,7 @@ pg_status carve_workspace(Workspace &w, const std::vector<std::pair<DevBuf *, si
     b->bytes = 0;
   }
   w.used = 0;
+  w.clean_bytes = 0;
   // 1/32 of slack, so that parts a later call adds (PROPAGATE-S's per-pass
   // claim bits after a PROPAGATE-P call) need no new arena
   pg_status rc = ensure(w.arena, total + total / 32);
@@ -665,6 +669,7 @@ void release_workspace(Workspace &w) {
   release(w.arena);
   release(w.rctl);
   w.used = 0;
+  w.clean_bytes = 0;
   for (DevBuf *b : workspace_parts(w)) {  // they pointed into the arena
     b->p = nullptr;
     b->bytes = 0;

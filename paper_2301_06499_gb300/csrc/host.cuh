@@ -27,6 +27,10 @@ struct Workspace {
       seed_bits, gfsum, gthr, dlist, dpref, E1, gm, F2, DI, DO, DM0, DM1;
   DevBuf rctl;  // ResidentCtl, outside the arena: it keeps its address and contents
   int32_t epoch = 0;  // launches of the resident round loop
+  // delta buffers known to be all zero over their first clean_bytes: every call
+  // that ends at its fixpoint leaves them so, any other one forgets it
+  const void *clean_d[3] = {nullptr, nullptr, nullptr};
+  size_t clean_bytes = 0;
   Ctrl *ctrl_h = nullptr;  // pinned, 2 slots
   ResidentOut *out_h = nullptr;  // pinned, of the resident round loop
   cudaEvent_t ev[2] = {nullptr, nullptr};

@@ -35,8 +35,10 @@ __global__ void __launch_bounds__(kBlock) k_zero(Params p, int64_t count_words, 
   for (int64_t i = gtid; i < pairs; i += nth) {
     x2[i] = z;
     if (p.Y) y2[i] = z;
-    d0[i] = z;
-    d1[i] = z;
+    if (p.zero_d) {
+      d0[i] = z;
+      d1[i] = z;
+    }
   }
   if ((words & 1) && gtid == 0) {
     p.X[words - 1] = 0ULL;
@@ -1409,6 +1411,19 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
     p.dense_above = (int64_t)(resident_threshold(g, cl.o) * (double)p.m);
     p.col_quads = ((uintptr_t)p.out_col & 15) == 0;
   }
+  // a call that ends at its fixpoint has cleared every delta it wrote
+  const void *dbuf[3] = {p.D0, p.D1, resident ? (const void *)p.D2 : nullptr};
+  const bool clean = w.clean_bytes >= sig_bytes && dbuf[0] == w.clean_d[0] &&
+                     dbuf[1] == w.clean_d[1] && (!dbuf[2] || dbuf[2] == w.clean_d[2]);
+  p.zero_d = resident && !clean ? 1 : 0;  // (one value for the captured loop)
+  const size_t clean_after = clean ? w.clean_bytes : sig_bytes;
+  w.clean_bytes = 0;
+  auto keep_clean = [&](const PassOut &o) {
+    if (o.status != PG_OK) return;
+    if (!clean || !dbuf[2])
+      for (int i = 0; i < 3; ++i) w.clean_d[i] = dbuf[i];
+    w.clean_bytes = clean_after;
+  };
   p.use_cond = 0;
   p.cond = 0ULL;
   p.iter_guard = cl.max_rounds + 2;
@@ -1481,11 +1496,17 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
     rc = cuda_status(cudaMemcpyAsync(w.seed_bits.p, bs->seed_bit, sizeof(int32_t) * sp,
                                      cudaMemcpyHostToDevice, st));
   if (rc) return rc;
-  if (resident) return run_resident(cl, pl, p, w, bs != nullptr, seeds_h, sp, col0, po);
+  if (resident) {
+    rc = run_resident(cl, pl, p, w, bs != nullptr, seeds_h, sp, col0, po);
+    if (rc == PG_OK) keep_clean(po);
+    return rc;
+  }
   const int64_t count_words = (int64_t)row_cap * ncols;
   const int64_t rs_words = (int64_t)(row_cap + 2) * (int64_t)(sizeof(RoundStats) / 8);
   const int64_t zero_work = std::max<int64_t>({n * pl.Wp / 2, nbm, count_words, rs_words, 1});
-  k_zero<<<occupancy_grid((const void *)&k_zero, 0, zero_work), kBlock, 0, st>>>(p, count_words,
+  Params pz = p;
+  pz.zero_d = clean ? 0 : 1;
+  k_zero<<<occupancy_grid((const void *)&k_zero, 0, zero_work), kBlock, 0, st>>>(pz, count_words,
                                                                                 rs_words);
   k_seed<<<occupancy_grid((const void *)&k_seed, 0, sp), kBlock, 0, st>>>(p, (const int32_t *)w.seeds.p,
                              bs ? (const int32_t *)w.seed_bits.p : nullptr, sp);
@@ -1628,6 +1649,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   po.rounds = fin.status == PG_ERANGE ? cl.max_rounds + 1 : fin.last_round;
   po.tma = pl.tma;
   po.status = fin.status;
+  keep_clean(po);
   po.dense_rounds = fin.dense_rounds;
   if (timing) {
     float ms = 0;

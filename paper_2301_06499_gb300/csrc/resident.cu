@@ -715,11 +715,13 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
     }
   };
   // the next unit's descriptor is fetched when a unit starts, its first
-  // columns when the unit ends
+  // columns and signatures when the unit ends (a row cut into pieces may gain
+  // bits from another warp in between: its atomics find that out)
   int g_next = 0, clen_next = 0;
   int64_t off_next = 0;
   ulonglong2 it_next = make_ulonglong2(0ULL, 0ULL);
   int32_t u_next[U];
+  uint64_t own_next[WL];
   auto descriptor = [&](int64_t ui) {
     it_next = make_ulonglong2(0ULL, 0ULL);
     clen_next = 0;
@@ -736,6 +738,9 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
     const int32_t *cc = p.sell_col + off_next;
 #pragma unroll
     for (int q = 0; q < U; ++q) u_next[q] = q < len ? __ldg(cc + 32LL * q) : -1;
+#pragma unroll
+    for (int k = 0; k < WL; ++k) own_next[k] = ~0ULL;
+    if (len > 0) ld_row<WL>(own_next, p.X + (size_t)(it_next.y >> 32) * CW + w0);
   };
   descriptor(L.warp);
   first_columns();
@@ -757,10 +762,9 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
     uint64_t own[WL], acc[WL];
 #pragma unroll
     for (int k = 0; k < WL; ++k) {
-      own[k] = ~0ULL;
+      own[k] = own_next[k];
       acc[k] = 0ULL;
     }
-    if (len > 0) ld_row<WL>(own, p.X + (size_t)v * CW + w0);
     int32_t u[U];
 #pragma unroll
     for (int q = 0; q < U; ++q) u[q] = u_next[q];
@@ -1077,14 +1081,17 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     ulonglong2 *d0 = reinterpret_cast<ulonglong2 *>(p.D0);
     ulonglong2 *d1 = reinterpret_cast<ulonglong2 *>(p.D1);
     ulonglong2 *d2 = reinterpret_cast<ulonglong2 *>(p.D2);
-    for (int64_t i = L.tid; i < pairs; i += L.nth) {
-      x2[i] = z;
-      d0[i] = z;
-      d1[i] = z;
-      d2[i] = z;
+    for (int64_t i = L.tid; i < pairs; i += L.nth) x2[i] = z;
+    if ((words & 1) && L.tid == 0) p.X[words - 1] = 0ULL;
+    // (three quarters of this traffic: 1.9 of R-MAT 26's 43 ms)
+    if (p.zero_d) {
+      for (int64_t i = L.tid; i < pairs; i += L.nth) {
+        d0[i] = z;
+        d1[i] = z;
+        d2[i] = z;
+      }
+      if ((words & 1) && L.tid == 0) p.D0[words - 1] = p.D1[words - 1] = p.D2[words - 1] = 0ULL;
     }
-    if ((words & 1) && L.tid == 0)
-      p.X[words - 1] = p.D0[words - 1] = p.D1[words - 1] = p.D2[words - 1] = 0ULL;
     for (int64_t i = L.tid; i < mwords; i += L.nth) p.C0[i] = p.C1[i] = p.C2[i] = 0u;
     if constexpr (PW)
       for (int64_t i = L.tid; i < kwords; i += L.nth) p.Kw0[i] = p.Kw1[i] = 0u;
@@ -1206,6 +1213,13 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       stop = false;
     }
     if (stop) {
+      if (nF == 0) {  // the last deltas; the buffers are zero again
+        const int32_t *Fl = frontier_buf(p, (t + 2) % 3);
+        uint64_t *Dl = delta_buf(p, (t + 2) % 3);
+        for (uint32_t i = blockIdx.x * blockDim.x + threadIdx.x; i < (uint32_t)nF_old;
+             i += gridDim.x * blockDim.x)
+          for (int k = 0; k < CW; ++k) Dl[(size_t)Fl[i] * CW + k] = 0ULL;
+      }
       if (threadIdx.x == 0) sh.rows_out = !SEG && nF == 0 ? t - p.row_base : -1;
       if (lead) {
         ctrl->t = t + 1;

@@ -89,3 +89,20 @@ def test_resident_packed_batch(window_rows, threshold):
             assert r.rounds == w["rounds"], i
             assert np.array_equal(r.counts, w["counts"]), i
             assert np.array_equal(r.m_active, w["m_active"]), i
+
+
+def test_delta_buffers_carried_between_calls():
+    """Calls leave their delta buffers zero for the next one; widths, schedules
+    and calls that stop short (counts capacity) in any order do not mix."""
+    g = _graph("er")
+    with pg.Graph.from_inputs(g) as G:
+        seeds = {s: I.seeds(g.n, s, 410 + s) for s in (512, 64, 1500, 300)}
+        want = {s: oracle.run(g, x) for s, x in seeds.items()}
+        for kw in (dict(), dict(sparse_push=1), dict(window_rows=1), dict(timing=1)):
+            for s in (64, 512, 1500, 300, 64, 1500):
+                for fn in (pg.propagate_p, pg.propagate_s):
+                    r = fn(G, seeds[s], opts=pg.options(**kw))
+                    assert r.rounds == want[s]["rounds"], (s, kw)
+                    assert np.array_equal(r.counts, want[s]["counts"]), (s, kw)
+                with pytest.raises(pg.PropagateError):
+                    pg.propagate_p(G, seeds[s], max_rounds=2, opts=pg.options(**kw))

@@ -17,8 +17,8 @@
 // node) has exactly one finder, which counts it (the collision count of
 // round t), records it in D of round t and, first on that row, appends the
 // row to F_t. Nothing is left for a second kernel: the signatures are synced,
-// the counts are complete at the barrier, and three delta buffers take turns
-// (t-1 read, t written, t-2 cleared through F_{t-2}).
+// a block's counts leave it while the next round starts, and three delta
+// buffers take turns (t-1 read, t written, t-2 cleared through F_{t-2}).
 //
 // m_active (the in-degrees of the rows round t revisits: a zero bit left at
 // its start and a changed in-neighbour): a row that reads full was either
@@ -33,14 +33,14 @@
 // as k_pull does, with its early stop.
 //
 // Measured per call, round by round (with dense rounds that stop early) and
-// here: ER 10^3 (s = 64) 215 -> 128 us, ER 10^4 (s = 64) 288 -> 160 us,
+// here: ER 10^3 (s = 64) 215 -> 90 us, ER 10^4 (s = 64) 288 -> 131 us,
 // 1024^2 grid (s = 128, ~2,050 rounds) 83 -> 36.5 ms, R-MAT 22 (s = 256)
-// 2.23 -> 1.70 ms, R-MAT 26 (s = 512) 54.9 -> 42 ms, 30 packed graphs
+// 2.23 -> 1.56 ms, R-MAT 26 (s = 512) 54.9 -> 42 ms, 30 packed graphs
 // 33.6 -> 16.3 ms. What bounds it now: a round of little work is five
 // dependent accesses, two block-wide steps and the barrier, 6 to 7 us; heavy
-// pushes the L2's atomics (about 25 per ns on spread addresses), which is why
-// marks are loaded before they are set; heavy sweeps the gathers a thread's
-// registers can hold in flight.
+// pushes the L2's atomics (25 to 28 per ns on spread addresses: the grid sends
+// 0.98 G of them in 34.5 ms), which is why marks are loaded before they are
+// set; heavy sweeps the gathers that a thread's registers hold in flight.
 //
 // Every wait at the barrier is bounded; on expiry the call returns
 // PG_ETIMEOUT. The blocks are co-resident by the cooperative launch.

@@ -34,7 +34,8 @@ namespace pg {
 // sweeps a longer row in passes of 128 words (4 per lane, so that 16 loads
 // of four neighbours are in flight), re-reading the piece's columns (from
 // L1) in each pass.
-// Three resident blocks per SM (80 registers; four of 64 for rows of 32 words).
+// Three resident blocks per SM (80 registers; four of 64 for rows of 32 words):
+// at 88 words four blocks spill, 16.0 against 14.9 ms a call on ER 10^6.
 //
 // PW: PROPAGATE-S passes as the words of one signature; m_active is counted
 // per pass here, in dense and sparse rounds alike (see count_pass_words).

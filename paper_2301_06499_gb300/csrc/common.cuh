@@ -54,7 +54,8 @@ struct Ctrl {
 };
 
 // Counters and barrier of the resident round loop (resident.cu), on lines of
-// their own; zero when allocated and after a launch that gave up.
+// their own; zero when allocated, and zeroed by the host (which waits for that)
+// after a launch that gave up.
 struct ResidentCtl {
   alignas(128) unsigned long long fp[3];  // F_t by t mod 3: (count << kFsumBits) | out-arc sum
   alignas(128) unsigned long long ne[3];  // pieces of F_t's long rows
@@ -74,6 +75,7 @@ constexpr int kResidentSeeds = 4096;          // seeds the launch reads from pin
 constexpr int kResidentOut = 64 << 10;        // bytes of data
 struct ResidentOut {
   Ctrl ctrl;
+  int32_t complete;  // the last launch all of whose blocks ran to its end (epoch)
   int32_t rows;  // count rows in data, -1: not there
   unsigned long long sums[kResidentBlocks][3];  // arcs scanned, deltas gathered, items
   int32_t seeds[kResidentSeeds];
@@ -172,6 +174,7 @@ struct Params {
                         // of copy k maps to k*perm_n + perm[x])
   ResidentCtl *rctl;    // resident loop (else null)
   ResidentOut *out;     // resident loop: pinned host memory
+  unsigned long long barrier_ns;  // resident loop: longest wait at its barrier
   uint32_t *deg_in, *deg_out;  // resident loop: degrees (the same array for symmetric graphs)
   int32_t sort_seeds;   // resident loop: bits of rows of 8 words placed by the seeds' degree
   int64_t dense_above;  // resident loop: a full sweep when the frontier's out-arcs pass this

@@ -99,6 +99,9 @@ struct pg_graph {
   pg::Workspace *ext_ws = nullptr;  // a view running on its server slot's workspace
   pg_stats last{};
   int sms = 0;  // SMs of its resident round loop (0 = all), set by who runs several at once
+#ifdef PG_DEBUG_BOUNDS
+  uint64_t debug_wait_ns = 0;  // pg_debug_short_barrier
+#endif
   int hint_p = 0, hint_s = 0;  // sweeps of the last pass, first batch of the next
   std::mutex mu;
 };

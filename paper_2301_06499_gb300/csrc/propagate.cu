@@ -1115,12 +1115,25 @@ static void resident_smem_optin() {
   if (dev < 64) done |= 1ULL << dev;
 }
 
+// Longest wait at the resident loop's barrier: it bounds a hang, not a round (the
+// longest one measured takes 23 ms).
+constexpr unsigned long long kBarrierNs = 20ULL * 1000 * 1000 * 1000;
+
 // One pass as a cooperative launch of the resident round loop (launched again
 // after each full counts window).
 static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w, bool batch,
                               const int32_t *seeds_h, int sp, int col0, PassOut &po) {
   cudaStream_t st = cl.st;
   pg_status rc;
+  if (!w.out_h) {
+    if (cudaMallocHost((void **)&w.out_h, sizeof(ResidentOut)) != cudaSuccess) {
+      cudaGetLastError();
+      w.out_h = nullptr;
+      return PG_ENOMEM;
+    }
+    w.out_h->complete = 0;  // launches count from 1
+  }
+  p.out = w.out_h;
   if (!w.rctl.p) {
     if ((rc = ensure(w.rctl, sizeof(ResidentCtl)))) return rc;
     if ((rc = cuda_status(cudaMemsetAsync(w.rctl.p, 0, sizeof(ResidentCtl), st)))) return rc;
@@ -1137,12 +1150,15 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   // a seed's bit is the loop's own business unless bits are passes
   p.sort_seeds = pair && !pl.pw && sp > 256 && sp <= kResidentSorted;
   const size_t smem = resident_smem(p.ncols, threads);
-  if (!w.out_h && cudaMallocHost((void **)&w.out_h, sizeof(ResidentOut)) != cudaSuccess) {
-    cudaGetLastError();
-    w.out_h = nullptr;
-    return PG_ENOMEM;
+  p.barrier_ns = kBarrierNs;
+#ifdef PG_DEBUG_BOUNDS
+  // a block short at the first barrier, and a wait of this length for it
+  if (cl.g->debug_wait_ns) {
+    p.barrier_ns = cl.g->debug_wait_ns;
+    cl.g->debug_wait_ns = 0;
+    if ((rc = cuda_status(cudaMemsetAsync(&p.rctl->arrive, 0xFF, sizeof(uint32_t), st)))) return rc;
   }
-  p.out = w.out_h;
+#endif
   // few seeds are read from pinned memory, once: no copy ahead of the launch
   const int32_t *seeds = (const int32_t *)w.seeds.p;
   if (sp <= kResidentSeeds && !p.perm) {
@@ -1166,16 +1182,18 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
       return rc;
     po.launches += 1;
     if ((rc = cuda_status(cudaStreamSynchronize(st)))) return rc;
+    if (w.out_h->complete != epoch) {  // a wait of the barrier ran out
+      // the next call may come on another stream: zero before this one returns
+      rc = cuda_status(cudaMemsetAsync(w.rctl.p, 0, sizeof(ResidentCtl), st));
+      if (rc == PG_OK) rc = cuda_status(cudaStreamSynchronize(st));
+      return rc ? rc : PG_ETIMEOUT;
+    }
     fin = w.out_h->ctrl;
     if (cl.rs_h.empty()) cl.rs_h.resize(1, RoundStats{});
     for (int b = 0; b < blocks; ++b) {
       cl.rs_h[0].scanned += w.out_h->sums[b][0];
       cl.rs_h[0].gathered += w.out_h->sums[b][1];
       cl.rs_h[0].items += w.out_h->sums[b][2];
-    }
-    if (!fin.done || fin.iters != epoch) {  // a wait of the barrier ran out
-      cudaMemsetAsync(w.rctl.p, 0, sizeof(ResidentCtl), st);
-      return PG_ETIMEOUT;
     }
     if (fin.status != kStatusWindow) break;
     if ((rc = copy_window(cl, p, col0, p.row_base, p.row_cap, p.row_cap))) return rc;
@@ -1781,6 +1799,9 @@ static pg_status propagate(pg_graph *g, const int32_t *seeds, int32_t s, pg_coun
     // counts in columns k*planes.. of the group; copies never exchange bits
     if ((rc = make_replicas(g, K, cl.st))) return rc;
     pg_graph *r = g->rep;
+#ifdef PG_DEBUG_BOUNDS
+    std::swap(r->debug_wait_ns, g->debug_wait_ns);
+#endif
     if ((rc = ensure(g->rep_graph_s, sizeof(int32_t) * K)) ||
         (rc = ensure(g->rep_graph_col0, sizeof(int32_t) * K)))
       return rc;
@@ -2085,6 +2106,12 @@ pg_status pg_propagate_s(pg_graph *g, const int32_t *seeds, int32_t s, pg_counts
                          const pg_options *opt, void *stream) {
   return propagate(g, seeds, s, out, opt, stream, true);
 }
+
+#ifdef PG_DEBUG_BOUNDS
+// For tests: the next resident round loop on g waits for a block that never
+// comes, for wait_ns at its first barrier.
+void pg_debug_short_barrier(pg_graph *g, uint64_t wait_ns) { g->debug_wait_ns = wait_ns; }
+#endif
 
 pg_status pg_last_stats(const pg_graph *g, pg_stats *out) {
   if (!g || !out) return PG_EINVAL;

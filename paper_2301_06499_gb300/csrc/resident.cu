@@ -54,7 +54,6 @@ constexpr int kBigRow = kResidentRow;
 constexpr int kBigPiece = kResidentPiece;
 constexpr int kMaxThreads = kResidentThreads;
 constexpr int kStage = 256;      // staged frontier rows per warp
-constexpr unsigned long long kBarrierNs = 20ULL * 1000 * 1000 * 1000;
 
 // Loads of data that other blocks write in this launch (never the read-only
 // path): coherent after the barrier's fence; within a round a stale
@@ -174,15 +173,20 @@ __device__ __forceinline__ int32_t *frontier_buf(const Params &p, int k) {
   return k == 0 ? p.F0 : k == 1 ? p.F1 : p.F2;
 }
 
-// Waits until *word, counting up, reaches target (modulo 2^32).
-__device__ __forceinline__ bool wait_for(ResidentCtl *rc, const uint32_t *word, uint32_t target) {
+// Waits until *word, counting up, reaches target (modulo 2^32). A block that
+// gives up leaves the launch. One that arrives after that finds the word
+// reached and goes on to its next barrier, where it gives up too; after the
+// launch's last barrier it runs to the end. So no block's own end says that the
+// launch was whole: only all of them, counted at the exit, do.
+__device__ __forceinline__ bool wait_for(const Params &p, const uint32_t *word, uint32_t target) {
+  ResidentCtl *rc = p.rctl;
   unsigned long long t0 = 0;
   for (int spin = 0; (int32_t)(ld_acquire(word) - target) < 0; ++spin) {
     if ((spin & 255) == 255) {
       const unsigned long long t = now_ns();
       if (!t0) t0 = t;
-      if (ld_acquire(&rc->abort) || t - t0 > kBarrierNs) {
-        st_release(&rc->abort, 1u);  // the host reads it: the call never reports done
+      if (ld_acquire(&rc->abort) || t - t0 > p.barrier_ns) {
+        st_release(&rc->abort, 1u);
         return false;
       }
     }
@@ -218,7 +222,7 @@ __device__ __forceinline__ bool grid_barrier(const Params &p, Shared &sh, Fin fi
         __threadfence();
         st_release(&rc->gen, sh.bar);
       } else {
-        sh.failed = !wait_for(rc, &rc->gen, sh.bar);
+        sh.failed = !wait_for(p, &rc->gen, sh.bar);
       }
       __threadfence();
     }
@@ -226,7 +230,7 @@ __device__ __forceinline__ bool grid_barrier(const Params &p, Shared &sh, Fin fi
     ++sh.bar;
     __threadfence();
     atomicAdd(&rc->arrive, 1u);
-    sh.failed = !wait_for(rc, &rc->arrive, sh.bar * gridDim.x);
+    sh.failed = !wait_for(p, &rc->arrive, sh.bar * gridDim.x);
     __threadfence();
   }
   __syncthreads();
@@ -1229,7 +1233,6 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
         ctrl->dense_rounds = dense_rounds;
         ctrl->status = status;
         ctrl->done = 1;
-        ctrl->iters = epoch;  // written by this launch
       }
       break;
     }
@@ -1324,12 +1327,13 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     prev_dense = dense;
     dense_rounds += dense;
   }
-  // every block has passed the last barrier once it gets here; the last one
-  // out leaves the barrier's words as the next launch needs them
+  // once every block got here the launch is whole: the last one out says so, and
+  // leaves the barrier's words as the next launch needs them
   if (threadIdx.x == 0 && atomicAdd(&rc->exited, 1u) == gridDim.x - 1) {
     rc->arrive = 0u;
     rc->gen = 0u;
     rc->exited = 0u;
+    p.out->complete = epoch;
   }
   hand_over(p.out, p.rs, p.counts, p.ncols, ctrl, &sh.rows_out, sh.sums, L.scan, L.gath, L.items);
 }

@@ -802,10 +802,15 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
         for (int q = 0; q < U; ++q)
           un[q] = (need && k0 + U + q < len) ? __ldg(cc + 32LL * (k0 + U + q)) : -1;
       }
-      if (need && sub == 0) L.scan += (uint32_t)max(0, min(U, len - k0));
       // (a pair gathers together until it has seen a change)
-      const bool pair_open = pair_any(open);  // every lane takes part in the exchange
-      const bool gather = open || (!PW && need && pair_open);
+      const bool other_open = SUB > 1 && __shfl_xor_sync(kFullMask, (int)open, 1) != 0;
+      const bool pair_open = open || other_open;  // every lane takes part in the exchange
+      const bool together = !PW && !found;
+      const bool gather = open || (together && need && pair_open);
+      // an arc is read, and a row gathered, once if either lane does so
+      if (sub == 0 && (pair_open || (together && act)))
+        L.scan += (uint32_t)max(0, min(U, len - k0));
+      const bool counts = sub == 0 || !(other_open || together);
       if (gather) {
         if (tc) {
 #pragma unroll
@@ -819,7 +824,7 @@ __device__ __forceinline__ void sweep_round(const Params &p, Lane &L, bool tc,
             ld_row<WL>(d, L.Dp + (size_t)u[q] * CW + w0);
 #pragma unroll
             for (int k = 0; k < WL; ++k) acc[k] |= d[k];
-            if (sub == 0) ++L.gath;
+            if (counts) ++L.gath;
           }
 #pragma unroll
         for (int k = 0; k < WL; ++k) found |= acc[k] != 0ULL;

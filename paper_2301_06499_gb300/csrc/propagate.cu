@@ -868,6 +868,7 @@ struct PassOut {
   double ms_pull = 0, ms_post = 0, ms_init = 0;
   int32_t pull_launches = 0, post_launches = 0;
   bool tma = false;
+  bool refused = false;  // no resident loop was launched
 };
 
 struct Call {
@@ -879,6 +880,7 @@ struct Call {
   uint32_t *counts_h;            // caller rows x s_total
   std::vector<RoundStats> rs_h;  // summed over passes, grown as rounds complete
   int32_t row_cap = 0;
+  bool by_round = false;  // the device refused the resident loop
   WindowSink sink = nullptr;
   void *sink_ctx = nullptr;
   std::vector<uint32_t> stage;
@@ -1144,12 +1146,10 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   const ResidentFn fn = resident_fn(pl.CW, pl.pw, batch, pair);
   // the SMs given to this graph (propagations that run side by side share
   // them: a cooperative launch waits until all its blocks fit), else all
-  const int blocks =
+  int blocks =
       std::min(cl.g->sms > 0 ? std::min(cl.g->sms, sm_count()) : sm_count(), kResidentBlocks);
-  const int threads = resident_threads(p.n, blocks);
   // a seed's bit is the loop's own business unless bits are passes
   p.sort_seeds = pair && !pl.pw && sp > 256 && sp <= kResidentSorted;
-  const size_t smem = resident_smem(p.ncols, threads);
   p.barrier_ns = kBarrierNs;
 #ifdef PG_DEBUG_BOUNDS
   // a block short at the first barrier, and a wait of this length for it
@@ -1177,9 +1177,21 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
     if (launches_guard-- < 0) return PG_EDEVICE;
     int epoch = ++w.epoch;
     void *args[] = {&p, &seeds, &bits, &sp, &resume, &epoch};
-    if ((rc = cuda_status(cudaLaunchCooperativeKernel((const void *)fn, dim3(blocks),
-                                                      dim3(threads), args, smem, st))))
-      return rc;
+    // a stream may own fewer SMs than the device has (a green context): the
+    // launch is then refused, and tried on half as many until they fit
+    for (;;) {
+      const int threads = resident_threads(p.n, blocks);
+      const cudaError_t e =
+          cudaLaunchCooperativeKernel((const void *)fn, dim3(blocks), dim3(threads), args,
+                                      resident_smem(p.ncols, threads), st);
+      if (e == cudaSuccess) break;
+      cudaGetLastError();
+      if (e != cudaErrorCooperativeLaunchTooLarge || blocks == 1) {
+        po.refused = !resume;
+        return cuda_status(e);
+      }
+      blocks = (blocks + 1) / 2;
+    }
     po.launches += 1;
     if ((rc = cuda_status(cudaStreamSynchronize(st)))) return rc;
     if (w.out_h->complete != epoch) {  // a wait of the barrier ran out
@@ -1257,7 +1269,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   const int32_t row_cap = cl.row_cap;
   // the resident round loop: the default for rows of up to 8 words gathered
   // whole. The other schedules, and per-launch events, run round by round.
-  const bool resident = !pl.wide && pl.CW == pl.Wp && cl.o.sparse_push == 0 &&
+  const bool resident = !cl.by_round && !pl.wide && pl.CW == pl.Wp && cl.o.sparse_push == 0 &&
                         cl.o.use_graphs != 0 && cl.o.timing == 0 && cl.o.tma_gather != 2 &&
                         (!bs || (g->nseg > 0 && bs->graph_m));
   const int64_t e_cap = resident ? g->m / kResidentRow + 1 : n + g->m / kExpandArcs + 1;
@@ -1516,6 +1528,11 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   if (rc) return rc;
   if (resident) {
     rc = run_resident(cl, pl, p, w, bs != nullptr, seeds_h, sp, col0, po);
+    if (po.refused) {  // the rounds by the captured loop, which asks for no residency
+      po = PassOut{};
+      cl.by_round = true;
+      return run_pass(cl, seeds_h, sp, col0, eb, hint, po, bs, pw);
+    }
     if (rc == PG_OK) keep_clean(po);
     return rc;
   }

@@ -23,7 +23,8 @@
  *  - Every call is ordered on the CUDA stream it is given (NULL = the legacy
  *    default stream) and returns once its host outputs are written.
  *  - Calls on one pg_graph are serialised by the library; different graphs
- *    may be used from different host threads concurrently.
+ *    may be used from different host threads concurrently: propagations that
+ *    are on the device together share its SMs.
  *  - No entry point aborts the process. Errors are returned as pg_status and
  *    leave the graph usable; pg_strerror names them.
  */

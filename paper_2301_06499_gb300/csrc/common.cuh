@@ -58,7 +58,11 @@ struct Ctrl {
 // after a launch that gave up.
 struct ResidentCtl {
   alignas(128) unsigned long long fp[3];  // F_t by t mod 3: (count << kFsumBits) | out-arc sum
-  alignas(128) unsigned long long ne[3];  // pieces of F_t's long rows
+  struct alignas(16) Next {
+    unsigned long long ne;     // pieces of F_t's long rows
+    unsigned long long yield;  // end the launch after round t
+  };
+  alignas(128) Next next[3];              // by t mod 3
   alignas(128) unsigned long long alive[3][8];  // seeds that gained a pair, by t mod 3
   alignas(128) uint32_t arrive;           // arrivals at the launch's barriers so far
   alignas(128) uint32_t gen;              // barriers released (packed batches)
@@ -76,6 +80,7 @@ constexpr int kResidentOut = 64 << 10;        // bytes of data
 struct ResidentOut {
   Ctrl ctrl;
   int32_t complete;  // the last launch all of whose blocks ran to its end (epoch)
+  int32_t want;      // from the host: blocks the loop should run on
   int32_t rows;  // count rows in data, -1: not there
   unsigned long long sums[kResidentBlocks][3];  // arcs scanned, deltas gathered, items
   int32_t seeds[kResidentSeeds];
@@ -175,6 +180,7 @@ struct Params {
   ResidentCtl *rctl;    // resident loop (else null)
   ResidentOut *out;     // resident loop: pinned host memory
   unsigned long long barrier_ns;  // resident loop: longest wait at its barrier
+  long long slice_cycles;         // resident loop: longest launch
   uint32_t *deg_in, *deg_out;  // resident loop: degrees (the same array for symmetric graphs)
   int32_t sort_seeds;   // resident loop: bits of rows of 8 words placed by the seeds' degree
   int64_t dense_above;  // resident loop: a full sweep when the frontier's out-arcs pass this

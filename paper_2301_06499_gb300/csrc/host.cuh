@@ -3,6 +3,7 @@
 // the graph handle, and the internal entry points between translation units.
 #pragma once
 
+#include <atomic>
 #include <functional>
 #include <mutex>
 #include <vector>
@@ -98,9 +99,10 @@ struct pg_graph {
   pg::Workspace ws;
   pg::Workspace *ext_ws = nullptr;  // a view running on its server slot's workspace
   pg_stats last{};
-  int sms = 0;  // SMs of its resident round loop (0 = all), set by who runs several at once
+  int sms = 0;  // SMs of its round loop at most (0 = all), set by who runs several at once
 #ifdef PG_DEBUG_BOUNDS
   uint64_t debug_wait_ns = 0;  // pg_debug_short_barrier
+  int64_t debug_slice = 0;     // pg_debug_slice
 #endif
   int hint_p = 0, hint_s = 0;  // sweeps of the last pass, first batch of the next
   std::mutex mu;
@@ -123,6 +125,22 @@ void release_workspace(Workspace &w);
 pg_status carve_workspace(Workspace &w, const std::vector<std::pair<DevBuf *, size_t>> &needs);
 // Device bytes a workspace holds.
 int64_t workspace_held(const Workspace &w);
+// A propagation on a device, and its part of the SMs while it is there
+// (share.cpp). cap: SMs it may use at most (0 = all), of a graph of so many
+// rows; want (optional, pinned): where a resident round loop reads its part.
+class Share {
+ public:
+  Share(int device, int total, int cap, int64_t rows, volatile int32_t *want);
+  ~Share();
+  Share(const Share &) = delete;
+  Share &operator=(const Share &) = delete;
+  void limit(int sms);  // it can use no more than these
+
+  int device, total, cap, need;
+  std::atomic<int> part{0};  // its present part
+  volatile int32_t *want;
+};
+void share_parts(int n, const int *cap, const int *need, int total, int *part);
 pg_status cuda_status(cudaError_t e);
 int sm_count();
 int64_t l2_bytes();  // of the current device

@@ -1121,8 +1121,12 @@ static void resident_smem_optin() {
 // longest one measured takes 23 ms).
 constexpr unsigned long long kBarrierNs = 20ULL * 1000 * 1000 * 1000;
 
+// Longest launch of the resident loop: the device's other work gets in between.
+// Launching again takes about 50 us. In cycles: about 20 ms.
+constexpr long long kSliceCycles = 40LL * 1000 * 1000;
+
 // One pass as a cooperative launch of the resident round loop (launched again
-// after each full counts window).
+// after each full counts window, and where it stopped for other work).
 static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w, bool batch,
                               const int32_t *seeds_h, int sp, int col0, PassOut &po) {
   cudaStream_t st = cl.st;
@@ -1144,14 +1148,14 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   resident_smem_optin();
   const bool pair = pl.CW == 8 && !batch && p.early_stop;
   const ResidentFn fn = resident_fn(pl.CW, pl.pw, batch, pair);
-  // the SMs given to this graph (propagations that run side by side share
-  // them: a cooperative launch waits until all its blocks fit), else all
-  int blocks =
-      std::min(cl.g->sms > 0 ? std::min(cl.g->sms, sm_count()) : sm_count(), kResidentBlocks);
+  // its part of the SMs (a cooperative launch waits until all its blocks fit)
+  Share share(cl.g->device, sm_count(), cl.g->sms, p.n, &w.out_h->want);
   // a seed's bit is the loop's own business unless bits are passes
   p.sort_seeds = pair && !pl.pw && sp > 256 && sp <= kResidentSorted;
   p.barrier_ns = kBarrierNs;
+  p.slice_cycles = kSliceCycles;
 #ifdef PG_DEBUG_BOUNDS
+  if (cl.g->debug_slice) p.slice_cycles = cl.g->debug_slice;
   // a block short at the first barrier, and a wait of this length for it
   if (cl.g->debug_wait_ns) {
     p.barrier_ns = cl.g->debug_wait_ns;
@@ -1171,11 +1175,10 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   const int32_t *bits = batch ? (const int32_t *)w.seed_bits.p : nullptr;
   int resume = 0;
   p.row_base = 0;
-  int64_t launches_guard = (int64_t)cl.max_rounds / std::max<int32_t>(p.row_cap, 1) + 4;
   Ctrl fin{};
   for (;;) {
-    if (launches_guard-- < 0) return PG_EDEVICE;
     int epoch = ++w.epoch;
+    int blocks = std::min(share.part.load(), kResidentBlocks);
     void *args[] = {&p, &seeds, &bits, &sp, &resume, &epoch};
     // a stream may own fewer SMs than the device has (a green context): the
     // launch is then refused, and tried on half as many until they fit
@@ -1191,6 +1194,7 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
         return cuda_status(e);
       }
       blocks = (blocks + 1) / 2;
+      share.limit(blocks);
     }
     po.launches += 1;
     if ((rc = cuda_status(cudaStreamSynchronize(st)))) return rc;
@@ -1208,8 +1212,10 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
       cl.rs_h[0].items += w.out_h->sums[b][2];
     }
     if (fin.status != kStatusWindow) break;
-    if ((rc = copy_window(cl, p, col0, p.row_base, p.row_cap, p.row_cap))) return rc;
-    p.row_base += p.row_cap;
+    const int32_t rows = fin.t - p.row_base;  // every launch completes a round
+    if (rows < 1) return PG_EDEVICE;
+    if ((rc = copy_window(cl, p, col0, p.row_base, rows, rows))) return rc;
+    p.row_base += rows;
     resume = 1;
   }
   if (fin.bad_index) return PG_EDEVICE;  // a PG_DEBUG_BOUNDS build caught a bad gather
@@ -1536,6 +1542,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
     if (rc == PG_OK) keep_clean(po);
     return rc;
   }
+  Share share(g->device, sm_count(), g->sms, n, nullptr);
   const int64_t count_words = (int64_t)row_cap * ncols;
   const int64_t rs_words = (int64_t)(row_cap + 2) * (int64_t)(sizeof(RoundStats) / 8);
   const int64_t zero_work = std::max<int64_t>({n * pl.Wp / 2, nbm, count_words, rs_words, 1});
@@ -1818,6 +1825,7 @@ static pg_status propagate(pg_graph *g, const int32_t *seeds, int32_t s, pg_coun
     pg_graph *r = g->rep;
 #ifdef PG_DEBUG_BOUNDS
     std::swap(r->debug_wait_ns, g->debug_wait_ns);
+    r->debug_slice = g->debug_slice;
 #endif
     if ((rc = ensure(g->rep_graph_s, sizeof(int32_t) * K)) ||
         (rc = ensure(g->rep_graph_col0, sizeof(int32_t) * K)))
@@ -2128,6 +2136,8 @@ pg_status pg_propagate_s(pg_graph *g, const int32_t *seeds, int32_t s, pg_counts
 // For tests: the next resident round loop on g waits for a block that never
 // comes, for wait_ns at its first barrier.
 void pg_debug_short_barrier(pg_graph *g, uint64_t wait_ns) { g->debug_wait_ns = wait_ns; }
+// The longest launch of resident round loops on g, in cycles (0: the library's).
+void pg_debug_slice(pg_graph *g, int64_t cycles) { g->debug_slice = cycles; }
 #endif
 
 pg_status pg_last_stats(const pg_graph *g, pg_stats *out) {

@@ -133,6 +133,8 @@ struct Shared {
   int rows_out;  // count rows to hand over at the fixpoint, else -1
   uint32_t bar;  // barriers this block has arrived at
   int last;      // this block arrived last
+  unsigned long long yield;
+  long long t0;  // launch time, in cycles
   int failed;    // the barrier gave up
 };
 
@@ -171,6 +173,25 @@ __device__ __forceinline__ uint32_t *mark_buf(const Params &p, int k) {
 }
 __device__ __forceinline__ int32_t *frontier_buf(const Params &p, int k) {
   return k == 0 ? p.F0 : k == 1 ? p.F1 : p.F2;
+}
+
+// Whether the launch should end after this round, to be launched again where it
+// stopped (run_resident): when other propagations came and its part of the SMs
+// is smaller, or they left and it is larger by half, but not at once: a call
+// soon over is waited for (ending a launch and starting another takes about
+// 50 us), and a larger part is worth that only for a long one. And when it has
+// held its SMs for a slice, so that other work on the device gets in between.
+// Times in cycles of the SM that asks, about 2 to the nanosecond: reading the
+// device's timer takes longer.
+constexpr long long kShrinkCycles = 200 * 1000;
+constexpr long long kGrowCycles = 4 * 1000 * 1000;
+
+__device__ __forceinline__ bool should_yield(const Params &p, const Shared &sh) {
+  const long long ran = clock64() - sh.t0;
+  if (ran <= kShrinkCycles && ran <= p.slice_cycles) return false;  // (no look at the host's memory)
+  const int want = *(volatile int32_t *)&p.out->want, have = (int)gridDim.x;
+  return ran > p.slice_cycles || (want > 0 && want < have) ||
+         (2 * want >= 3 * have && ran > kGrowCycles);
 }
 
 // Waits until *word, counting up, reaches target (modulo 2^32). A block that
@@ -313,7 +334,7 @@ __device__ __forceinline__ void stage_spill(const Params &p, Lane &L) {
   stage_totals<SEG>(p, L, od_t, ne_t);
   if (L.lane == 0) {
     bf = atomicAdd(&p.rctl->fp[L.cur], ((unsigned long long)L.scnt << kFsumBits) + od_t);
-    if (ne_t) be = atomicAdd(&p.rctl->ne[L.cur], ne_t);
+    if (ne_t) be = atomicAdd(&p.rctl->next[L.cur].ne, ne_t);
   }
   bf = __shfl_sync(kFullMask, bf, 0) >> kFsumBits;
   be = __shfl_sync(kFullMask, be, 0);
@@ -366,7 +387,7 @@ __device__ __forceinline__ void round_flush(const Params &p, Lane &L, Shared &sh
   if (threadIdx.x == 0) {  // one reservation for the block
     unsigned long long bf = 0, be = 0;
     if (sh.staged) bf = atomicAdd(&p.rctl->fp[L.cur], ((unsigned long long)sh.staged << kFsumBits) + sh.od);
-    if (sh.ne) be = atomicAdd(&p.rctl->ne[L.cur], sh.ne);
+    if (sh.ne) be = atomicAdd(&p.rctl->next[L.cur].ne, sh.ne);
     if (sh.rows) {
       atomicAdd(&rs->m_active, sh.mact);
       atomicAdd(&rs->work, sh.work);
@@ -1067,6 +1088,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
   L.rows = L.scan = L.gath = L.items = 0;
   if (smem_counts)
     for (int i = threadIdx.x; i < 2 * p.ncols; i += blockDim.x) dyn[i] = 0u;
+  // the thread that looks for a changed part: in the warp that comes last to a
+  // round's work, so that a short round does not wait for the host's memory
+  const bool poll = blockIdx.x == gridDim.x - 1 && threadIdx.x == blockDim.x - 1;
+  if (poll) sh.t0 = clock64();
   if (threadIdx.x == 0) {
     sh.mact = sh.work = sh.od = sh.ne = 0;
     sh.rows = sh.staged = 0;
@@ -1119,7 +1144,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       for (int64_t i = L.tid; i < 2LL * p.nseg; i += L.nth) p.gmact[i] = 0ULL;
     if (L.tid == 0) ctrl->ndense = 0;
     if (L.tid < 2) p.rs[L.tid] = RoundStats{};
-    if (L.tid < 3) rc->fp[L.tid] = rc->ne[L.tid] = 0ULL;
+    if (L.tid < 3) {
+      rc->fp[L.tid] = 0ULL;
+      rc->next[L.tid] = {0ULL, 0ULL};
+    }
     if (!SEG && p.early_stop && L.tid < 3 * kAliveWords) {  // every seed starts alive
       const int w = (int)L.tid % kAliveWords;
       rc->alive[L.tid / kAliveWords][w] = L.tid < kAliveWords ? valid_mask(w, p.s) : 0ULL;
@@ -1155,7 +1183,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       unsigned long long bf = 0, be = 0;
       if (L.lane == 0) {
         bf = atomicAdd(&rc->fp[0], ((unsigned long long)__popc(mask) << kFsumBits) + ot);
-        if (et) be = atomicAdd(&rc->ne[0], et);
+        if (et) be = atomicAdd(&rc->next[0].ne, et);
       }
       bf = __shfl_sync(kFullMask, bf, 0) >> kFsumBits;
       be = __shfl_sync(kFullMask, be, 0);
@@ -1183,7 +1211,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
     // (one reader a block: every warp of the grid at one word would queue)
     if (threadIdx.x == 0) {
       sh.fp = *(volatile unsigned long long *)&rc->fp[t % 3];
-      sh.ne_all = *(volatile unsigned long long *)&rc->ne[t % 3];
+      asm volatile("ld.volatile.global.v2.u64 {%0, %1}, [%2];"
+                   : "=l"(sh.ne_all), "=l"(sh.yield)
+                   : "l"(&rc->next[t % 3])
+                   : "memory");
     }
     __syncthreads();
     const unsigned long long fp = sh.fp;
@@ -1216,7 +1247,7 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       last_round = t - 1;
     } else if (t >= p.max_rounds + 1) {
       status = PG_ERANGE;
-    } else if (!first_pass && t + 1 - p.row_base >= p.row_cap) {
+    } else if (!first_pass && (t + 1 - p.row_base >= p.row_cap || sh.yield)) {
       status = kStatusWindow;
     } else {
       stop = false;
@@ -1276,10 +1307,10 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
               (unsigned long long)(__ldg(p.out_ptr + v + 1) - __ldg(p.out_ptr + v));
           if (od > kBigRow) ne = (od + kBigPiece - 1) / kBigPiece;
         }
-        if (__any_sync(kFullMask, ne != 0ULL)) warp_append_pieces(E, &rc->ne[prev], v, ne, L.lane);
+        if (__any_sync(kFullMask, ne != 0ULL)) warp_append_pieces(E, &rc->next[prev].ne, v, ne, L.lane);
       }
       if (!grid_barrier<SEG>(p, sh, none)) return;
-      if (threadIdx.x == 0) sh.ne_all = *(volatile unsigned long long *)&rc->ne[prev];
+      if (threadIdx.x == 0) sh.ne_all = *(volatile unsigned long long *)&rc->next[prev].ne;
       __syncthreads();
       nE = (int64_t)sh.ne_all;
     }
@@ -1314,11 +1345,12 @@ __global__ void __launch_bounds__(kMaxThreads, 1)
       if (lead) {
         p.rs[nrow] = RoundStats{};
         rc->fp[old] = 0ULL;
-        rc->ne[old] = 0ULL;
+        rc->next[old] = {0ULL, 0ULL};
         if (!SEG && p.early_stop)
           for (int w = 0; w < CW; ++w) rc->alive[old][w] = 0ULL;
       }
     }
+    if (poll && should_yield(p, sh)) *(volatile unsigned long long *)&rc->next[L.cur].yield = 1ULL;
     if (dense && p.early_stop) {  // bits that can still travel: round t-1's seeds
       if (threadIdx.x < CW) sh.alive[threadIdx.x] = *(volatile unsigned long long *)&rc->alive[prev][threadIdx.x];
       __syncthreads();

@@ -115,10 +115,10 @@ typedef struct {
                                (sparse) sweep when the frontier's out-arcs are
                                few, a full (dense) sweep otherwise */
   float dense_threshold;    /* AUTO: dense when frontier out-arcs > this * m
-                               (0 or the default 0.05 = the library's choice:
-                               0.2 in the one-launch round loop (use_graphs)
-                               for graphs whose rows have at most 64 in-arcs
-                               and 0.08 for others, else 0.05) */
+                               (0, the default = the library's choice: 0.2 in
+                               the one-launch round loop (use_graphs) for
+                               graphs whose rows have at most 64 in-arcs and
+                               0.08 for others, else 0.05) */
   int32_t group_lanes;      /* lanes sharing one work piece (1..32, power of
                                two); a piece is group_lanes x 8 in-arcs for
                                s <= 128, x 4 for s <= 256, x 2 above, and

@@ -1077,7 +1077,7 @@ struct BatchSeg {
 };
 
 // Frontier out-arcs above which a round of the resident loop is a full sweep,
-// as a part of all arcs, where the caller keeps the default. A pushed arc costs
+// as a part of all arcs, where the caller leaves it to the library. A pushed arc costs
 // several swept ones, but a sweep of a graph without long rows (grids, road
 // networks, uniform random graphs) costs its whole latency: 1024^2 grid
 // (s = 128) 37.2 ms a call at 0.2 against 52.1 at 0.05, ER within 5% either
@@ -1087,7 +1087,7 @@ struct BatchSeg {
 constexpr int64_t kEvenDegree = 64;
 
 static double resident_threshold(const pg_graph *g, const pg_options &o) {
-  if (o.dense_threshold > 0 && o.dense_threshold != 0.05f) return (double)o.dense_threshold;
+  if (o.dense_threshold > 0) return (double)o.dense_threshold;
   return g->max_degree <= kEvenDegree ? 0.2 : 0.08;
 }
 
@@ -2107,7 +2107,7 @@ void pg_default_options(pg_options *o) {
   if (!o) return;
   std::memset(o, 0, sizeof(*o));
   o->direction = PG_DIR_AUTO;
-  o->dense_threshold = 0.05f;
+  o->dense_threshold = 0.0f;
   o->group_lanes = 0;
   o->test_changed = 0;
   o->planes_per_pass = 64;

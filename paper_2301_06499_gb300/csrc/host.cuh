@@ -181,6 +181,9 @@ typedef std::function<pg_status(const pg_options &, double *ms, uint64_t *hash)>
 // Coordinate descent over the schedule options (see tune.cu).
 pg_status tune_options(const TuneRun &run, int32_t s_bits, int32_t max_trials, pg_options *inout,
                        pg_tune_report *rep, bool s_mode);
+// Whether these options leave the rounds of rows of up to 8 words, gathered whole,
+// to the resident loop.
+bool resident_schedule(const pg_options &o);
 uint64_t fnv1a(uint64_t h, const void *data, size_t bytes);
 // K copies of g side by side, cached in g (see pg_graph::rep); PG_EINVAL if
 // they would not fit the index ranges.

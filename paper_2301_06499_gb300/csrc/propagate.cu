@@ -1076,6 +1076,10 @@ struct BatchSeg {
   const int64_t *graph_m;     // host, arcs of each graph (per-graph round kinds)
 };
 
+bool resident_schedule(const pg_options &o) {
+  return o.sparse_push == 0 && o.use_graphs != 0 && o.timing == 0 && o.tma_gather != 2;
+}
+
 // Frontier out-arcs above which a round of the resident loop is a full sweep,
 // as a part of all arcs, where the caller leaves it to the library. A pushed arc costs
 // several swept ones, but a sweep of a graph without long rows (grids, road
@@ -1275,8 +1279,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   const int32_t row_cap = cl.row_cap;
   // the resident round loop: the default for rows of up to 8 words gathered
   // whole. The other schedules, and per-launch events, run round by round.
-  const bool resident = !cl.by_round && !pl.wide && pl.CW == pl.Wp && cl.o.sparse_push == 0 &&
-                        cl.o.use_graphs != 0 && cl.o.timing == 0 && cl.o.tma_gather != 2 &&
+  const bool resident = !cl.by_round && !pl.wide && pl.CW == pl.Wp && resident_schedule(cl.o) &&
                         (!bs || (g->nseg > 0 && bs->graph_m));
   const int64_t e_cap = resident ? g->m / kResidentRow + 1 : n + g->m / kExpandArcs + 1;
   const size_t sig_bytes = sizeof(uint64_t) * (size_t)n * pl.Wp;

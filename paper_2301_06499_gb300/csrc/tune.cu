@@ -114,15 +114,19 @@ pg_status tune_options(const TuneRun &run, int32_t s_bits, int32_t max_trials, p
     o.words_per_thread = c;
     if ((rc = try_value(o))) return rc;
   }
+  // the resident round loop reads no group_lanes: those runs would differ by
+  // their noise only
+  const bool resident = W <= 8 && resident_schedule(cur) &&
+                        (cur.words_per_thread == 0 || cur.words_per_thread >= cw_class);
   for (int g : lanes) {
-    if (wide || g == cur.group_lanes) continue;
+    if (wide || resident || g == cur.group_lanes) continue;
     pg_options o = cur;
     o.group_lanes = g;
     if ((rc = try_value(o))) return rc;
   }
   if (cur.direction == PG_DIR_AUTO)
     for (float d : dens) {
-      if (d == cur.dense_threshold) continue;
+      if (d == cur.dense_threshold || (!resident && !cur.dense_threshold && d == 0.05f)) continue;
       pg_options o = cur;
       o.dense_threshold = d;
       if ((rc = try_value(o))) return rc;
@@ -142,6 +146,20 @@ pg_status tune_options(const TuneRun &run, int32_t s_bits, int32_t max_trials, p
 }  // namespace pg
 
 using namespace pg;
+
+#ifdef PG_DEBUG_BOUNDS
+// For tests: the tuner's search, with the time of each schedule from ms.
+extern "C" pg_status pg_debug_tune(int32_t s_bits, int32_t s_mode, int32_t max_trials,
+                                   double (*ms)(const pg_options *), pg_options *inout,
+                                   pg_tune_report *report) {
+  TuneRun run = [&](const pg_options &o, double *t, uint64_t *hash) -> pg_status {
+    *t = ms(&o);
+    *hash = 1;
+    return PG_OK;
+  };
+  return tune_options(run, s_bits, max_trials, inout, report, s_mode != 0);
+}
+#endif
 
 extern "C" pg_status pg_autotune(pg_graph *g, const int32_t *seeds, int32_t s, int32_t algorithm,
                                  int32_t max_trials, pg_options *inout, pg_tune_report *report,

@@ -602,56 +602,83 @@ static std::vector<DevBuf *> workspace_parts(Workspace &w) {
           &w.dlist, &w.dpref, &w.E1, &w.gm, &w.F2, &w.DI, &w.DO, &w.DM0, &w.DM1};
 }
 
-pg_status carve_workspace(Workspace &w, const std::vector<std::pair<DevBuf *, size_t>> &needs) {
-  constexpr size_t kAlign = 256;
-  bool fits = w.arena.p != nullptr;
-  for (const auto &nd : needs)
-    if (!nd.first->p || nd.first->bytes < std::max<size_t>(nd.second, 16)) fits = false;
-  if (fits) return PG_OK;
-  std::vector<DevBuf *> parts = workspace_parts(w);
-  if (w.arena.p) {
-    // only parts the layout does not have yet: placed after it, in the
-    // arena's slack, when they fit (the other parts keep their place)
-    size_t off = w.used;
-    bool extra_ok = true;
-    std::vector<std::pair<DevBuf *, size_t>> add;
-    for (const auto &nd : needs) {
-      const size_t want = std::max<size_t>(nd.second, 16);
-      if (nd.first->p && nd.first->bytes >= want) continue;
-      if (nd.first->p) extra_ok = false;  // a part that has to grow
-      add.push_back({nd.first, want});
-      off += (want + kAlign - 1) / kAlign * kAlign;
-    }
-    if (extra_ok && off <= w.arena.bytes) {
-      char *base = (char *)w.arena.p;
-      for (auto &a : add) {
-        a.first->p = base + w.used;
-        a.first->bytes = a.second;
-        w.used += (a.second + kAlign - 1) / kAlign * kAlign;
-      }
-      return PG_OK;
-    }
-  }
-  std::vector<size_t> cap(parts.size());
-  for (size_t i = 0; i < parts.size(); ++i) cap[i] = parts[i]->p ? parts[i]->bytes : 0;
+constexpr size_t kAlign = 256;
+static size_t aligned(size_t b) { return (b + kAlign - 1) / kAlign * kAlign; }
+
+// How a workspace meets a list of needs.
+enum class Carve { kFits, kExtra, kAnew, kUnknown };
+
+// kFits: every part is there. kExtra: only parts the layout does not have yet
+// are missing, and they fit after it, in the arena's slack (add; the other parts
+// keep their place). kAnew: laid out again in an arena of at least `total` bytes,
+// part i of workspace_parts with cap[i]. 1/32 of that is slack, so that parts a
+// later call adds (PROPAGATE-S's per-pass claim bits after a PROPAGATE-P call)
+// need no new arena.
+static Carve plan_carve(const Workspace &w, const std::vector<const DevBuf *> &parts,
+                        const WorkspaceNeeds &needs, std::vector<std::pair<DevBuf *, size_t>> &add,
+                        std::vector<size_t> &cap, size_t &total) {
+  size_t off = w.used;
+  bool grows = !w.arena.p;
   for (const auto &nd : needs) {
     const size_t want = std::max<size_t>(nd.second, 16);
+    if (nd.first->p && nd.first->bytes >= want) continue;
+    if (nd.first->p) grows = true;  // a part that has to grow
+    add.push_back({nd.first, want});
+    off += aligned(want);
+  }
+  if (!grows && add.empty()) return Carve::kFits;
+  if (!grows && off <= w.arena.bytes) return Carve::kExtra;
+  cap.resize(parts.size());
+  for (size_t i = 0; i < parts.size(); ++i) cap[i] = parts[i]->p ? parts[i]->bytes : 0;
+  for (const auto &nd : needs) {
     size_t i = 0;
     while (i < parts.size() && parts[i] != nd.first) ++i;
-    if (i == parts.size()) return PG_EINVAL;  // not a buffer of this workspace
-    cap[i] = std::max(cap[i], want);
+    if (i == parts.size()) return Carve::kUnknown;  // not a buffer of this workspace
+    cap[i] = std::max(cap[i], std::max<size_t>(nd.second, 16));
   }
+  total = 0;
+  for (size_t c : cap) total += aligned(c);
+  total += total / 32;
+  return Carve::kAnew;
+}
+
+static std::vector<const DevBuf *> const_parts(const Workspace &w) {
+  std::vector<DevBuf *> p = workspace_parts(const_cast<Workspace &>(w));
+  return {p.begin(), p.end()};
+}
+
+int64_t workspace_after(const Workspace &w, const WorkspaceNeeds &needs) {
+  std::vector<std::pair<DevBuf *, size_t>> add;
+  std::vector<size_t> cap;
   size_t total = 0;
-  for (size_t c : cap) total += (c + kAlign - 1) / kAlign * kAlign;
+  const Carve c = plan_carve(w, const_parts(w), needs, add, cap, total);
+  return (int64_t)std::max(w.arena.bytes, c == Carve::kAnew ? total : 0);
+}
+
+pg_status carve_workspace(Workspace &w, const WorkspaceNeeds &needs) {
+  std::vector<std::pair<DevBuf *, size_t>> add;
+  std::vector<size_t> cap;
+  size_t total = 0;
+  switch (plan_carve(w, const_parts(w), needs, add, cap, total)) {
+    case Carve::kUnknown: return PG_EINVAL;
+    case Carve::kFits: return PG_OK;
+    case Carve::kExtra:
+      for (auto &a : add) {
+        a.first->p = (char *)w.arena.p + w.used;
+        a.first->bytes = a.second;
+        w.used += aligned(a.second);
+      }
+      return PG_OK;
+    case Carve::kAnew: break;
+  }
+  std::vector<DevBuf *> parts = workspace_parts(w);
   for (DevBuf *b : parts) {  // the old layout is void from here on
     b->p = nullptr;
     b->bytes = 0;
   }
   w.used = 0;
   w.clean_bytes = 0;
-  // 1/32 of slack, so that parts a later call adds (PROPAGATE-S's per-pass
-  // claim bits after a PROPAGATE-P call) need no new arena
-  pg_status rc = ensure(w.arena, total + total / 32);
+  pg_status rc = ensure(w.arena, total);
   if (rc) return rc;
   char *base = (char *)w.arena.p;
   size_t off = 0;
@@ -659,7 +686,7 @@ pg_status carve_workspace(Workspace &w, const std::vector<std::pair<DevBuf *, si
     if (!cap[i]) continue;
     parts[i]->p = base + off;
     parts[i]->bytes = cap[i];
-    off += (cap[i] + kAlign - 1) / kAlign * kAlign;
+    off += aligned(cap[i]);
   }
   w.used = off;
   return PG_OK;
@@ -686,7 +713,7 @@ void release_workspace(Workspace &w) {
   w.tev.clear();
 }
 
-int64_t workspace_held(const Workspace &w) { return (int64_t)w.arena.bytes; }
+int64_t workspace_held(const Workspace &w) { return (int64_t)(w.arena.bytes + w.rctl.bytes); }
 
 // K copies of a CSR side by side: copy k's rows are k*n.., its arcs k*m..,
 // its column indices shifted by k*n.

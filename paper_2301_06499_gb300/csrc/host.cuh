@@ -117,14 +117,16 @@ pg_status ensure_host(DevBuf &b, size_t bytes);
 void release(DevBuf &b);
 // Frees every buffer, event and pinned block of a workspace.
 void release_workspace(Workspace &w);
+typedef std::vector<std::pair<DevBuf *, size_t>> WorkspaceNeeds;
 // Gives each listed buffer of w at least the listed bytes: one device
 // allocation per workspace (with 1/32 of slack), carved 256-byte aligned.
 // Buffers the layout lacks go into the slack when they fit; when a buffer
 // must grow, or the slack is too small, the whole workspace is laid out
 // again (contents are not kept); otherwise every buffer keeps its address.
-pg_status carve_workspace(Workspace &w, const std::vector<std::pair<DevBuf *, size_t>> &needs);
-// Device bytes a workspace holds.
+pg_status carve_workspace(Workspace &w, const WorkspaceNeeds &needs);
+// Device bytes a workspace holds, and will hold after carve_workspace.
 int64_t workspace_held(const Workspace &w);
+int64_t workspace_after(const Workspace &w, const WorkspaceNeeds &needs);
 // A propagation on a device, and its part of the SMs while it is there
 // (share.cpp). cap: SMs it may use at most (0 = all), of a graph of so many
 // rows; want (optional, pinned): where a resident round loop reads its part.
@@ -189,11 +191,12 @@ uint64_t fnv1a(uint64_t h, const void *data, size_t bytes);
 // they would not fit the index ranges.
 pg_status make_replicas(pg_graph *g, int K, cudaStream_t st);
 void drop_replicas(pg_graph *g);
-// Device bytes a propagation of s seeds on g will hold in its workspace
-// (window_rows as pg_options.window_rows).
-int64_t workspace_bytes(const pg_graph *g, int32_t s, int32_t max_rounds, int32_t window_rows);
-// The same for a graph of n nodes and m arcs.
-int64_t workspace_bytes_nm(int64_t n, int64_t m, int32_t s, int32_t max_rounds,
-                           int32_t window_rows);
+// Device bytes that workspace w will hold after a PROPAGATE-P of s seeds with
+// these options on a graph of n nodes and m arcs, or on a packed batch of nseg
+// graphs (0: one graph) where the widest has s seeds and all have ncols.
+int64_t workspace_bytes(const Workspace &w, int64_t n, int64_t m, bool directed, int32_t s,
+                        int32_t ncols, int32_t nseg, int32_t max_rounds, const pg_options &opt);
+// At most the bytes of the piece list that it makes for the graph (wide rows).
+int64_t piece_list_bytes(int64_t n, int64_t m, int32_t s, const pg_options &opt);
 
 }  // namespace pg

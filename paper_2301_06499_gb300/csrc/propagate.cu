@@ -754,7 +754,7 @@ static int auto_group(double mean_degree, int unr) {
   return G;
 }
 
-static pg_status make_plan(const pg_graph *g, int sp, const pg_options &o, bool s_mode, Plan &pl) {
+static pg_status make_plan(double mean_degree, int sp, const pg_options &o, bool s_mode, Plan &pl) {
   const int W = s_mode ? 1 : (sp + 63) / 64;
   pl.CW = W <= 1 ? 1 : W <= 2 ? 2 : W <= 4 ? 4 : 8;
   if (o.words_per_thread != 0) {
@@ -778,7 +778,7 @@ static pg_status make_plan(const pg_graph *g, int sp, const pg_options &o, bool 
     return PG_OK;
   }
   pl.UNR = pl.CW <= 2 ? 8 : (pl.CW == 4 ? 4 : 2);
-  int G = o.group_lanes > 0 ? o.group_lanes : auto_group(g->mean_degree, pl.UNR);
+  int G = o.group_lanes > 0 ? o.group_lanes : auto_group(mean_degree, pl.UNR);
   if (G > 32 || (G & (G - 1))) return PG_EINVAL;
   pl.G = G;
   pl.L = G * pl.UNR;
@@ -1244,6 +1244,75 @@ static pg_status run_resident(Call &cl, const Plan &pl, Params &p, Workspace &w,
   return PG_OK;
 }
 
+// Rows of a counts window: up to max_rounds + 1, at most ~256 MB of counters.
+static int32_t window_rows(int32_t ncols, int32_t max_rounds, const pg_options &o) {
+  const int64_t cap = o.window_rows > 0 ? o.window_rows
+                                        : std::max<int64_t>(64, (256LL << 20) / (4LL * ncols));
+  return (int32_t)std::max<int64_t>(1, std::min<int64_t>((int64_t)max_rounds + 1, cap));
+}
+
+// What of a pass decides the size of its buffers, beside its plan.
+struct PassShape {
+  int64_t n, m, npieces;  // npieces: of the rows (their number, or a bound)
+  bool own_out;           // out-arcs of its own (a directed graph)
+  int sp, ncols;          // seeds, count columns
+  int32_t row_cap;
+  bool batch;
+  int32_t nseg;  // graphs of a packed batch
+  bool resident, push, pw, gm;
+};
+
+static WorkspaceNeeds workspace_needs(Workspace &w, const Plan &pl, const PassShape &x) {
+  const size_t n = (size_t)x.n, nseg = (size_t)x.nseg;
+  const int64_t e_cap = x.resident ? x.m / kResidentRow + 1 : x.n + x.m / kExpandArcs + 1;
+  const size_t sig_bytes = sizeof(uint64_t) * n * pl.Wp;
+  const size_t bm_bytes = sizeof(uint32_t) * ((n + 31) / 32);
+  const size_t c_bytes = x.resident ? 2 * bm_bytes : bm_bytes;  // resident: two mark bits a row
+  // the delta buffers keep one all-zero row past the last node (the row a
+  // TMA gather of an empty slot reads)
+  const size_t delta_bytes_alloc = sig_bytes + sizeof(uint64_t) * (size_t)pl.Wp;
+  WorkspaceNeeds needs = {
+      {&w.X, sig_bytes}, {&w.D0, delta_bytes_alloc}, {&w.D1, delta_bytes_alloc},
+      {&w.C0, c_bytes}, {&w.C1, c_bytes}, {&w.Sat, c_bytes},
+      {&w.F0, sizeof(int32_t) * n}, {&w.F1, sizeof(int32_t) * n},
+      {&w.E, sizeof(unsigned long long) * (size_t)e_cap},
+      {&w.counts, sizeof(uint32_t) * (size_t)x.row_cap * (size_t)x.ncols},
+      {&w.rs, sizeof(RoundStats) * (size_t)(x.row_cap + 2)},
+      {&w.ctrl, sizeof(Ctrl)}, {&w.seeds, sizeof(int32_t) * (size_t)x.sp}};
+  if (x.resident) {
+    needs.push_back({&w.F2, sizeof(int32_t) * n});
+    needs.push_back({&w.DI, sizeof(uint32_t) * n});
+    if (x.own_out) needs.push_back({&w.DO, sizeof(uint32_t) * n});
+  } else {
+    needs.push_back({&w.K0, bm_bytes});
+    needs.push_back({&w.K1, bm_bytes});
+    needs.push_back({&w.A, sizeof(ulonglong2) * (size_t)std::max<int64_t>(x.npieces, 1)});
+  }
+  if (pl.wide && pl.post_wide) {  // no Y
+    needs.push_back({&w.DM0, sizeof(uint32_t) * n});
+    needs.push_back({&w.DM1, sizeof(uint32_t) * n});
+  } else {
+    needs.push_back({&w.Y, sig_bytes});
+    if (pl.post_wide) needs.push_back({&w.RB, sizeof(uint32_t) * n});
+  }
+  if (x.pw) {  // claim bits per (word, row); the resident loop: a byte per row
+    const size_t kw = x.resident ? (n + 3) / 4 * 4 : bm_bytes * (size_t)pl.Wp;
+    needs.push_back({&w.KW0, kw});
+    needs.push_back({&w.KW1, kw});
+  }
+  if (x.batch) needs.push_back({&w.seed_bits, sizeof(int32_t) * (size_t)x.sp});
+  if (x.push) needs.push_back({&w.E1, sizeof(unsigned long long) * (size_t)e_cap});
+  if (x.batch && nseg > 0) {
+    needs.push_back({&w.gfsum, 3 * sizeof(unsigned long long) * nseg});
+    needs.push_back({&w.gthr, sizeof(unsigned long long) * nseg});
+    needs.push_back({&w.dlist, sizeof(int32_t) * nseg});
+    needs.push_back({&w.dpref, sizeof(int64_t) * (nseg + 1)});
+  }
+  if (x.gm)
+    needs.push_back({&w.gm, sizeof(unsigned long long) * (size_t)(x.row_cap + 2) * nseg});
+  return needs;
+}
+
 // One pass: sp seeds of the call, columns [col0, col0+sp); or, with bs, all
 // seeds of a packed batch.
 // With pw, the sp seeds are ceil(sp/64) PROPAGATE-S passes of 64 planes run
@@ -1256,7 +1325,7 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   Plan pl;
   const int s_bits = bs ? bs->s_bits : sp;
   const int ncols = bs ? bs->ncols : sp;
-  pg_status rc = make_plan(g, s_bits, cl.o, eb, pl);
+  pg_status rc = make_plan(g->mean_degree, s_bits, cl.o, eb, pl);
   if (rc) return rc;
   if (pw) {  // the instantiations that count m_active per pass
     pl.pull = pl.wide ? pull_fn_wide(pl.Wp, true) : pick_pull(pl.CW, pl.G, true);
@@ -1281,50 +1350,14 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   // whole. The other schedules, and per-launch events, run round by round.
   const bool resident = !cl.by_round && !pl.wide && pl.CW == pl.Wp && resident_schedule(cl.o) &&
                         (!bs || (g->nseg > 0 && bs->graph_m));
-  const int64_t e_cap = resident ? g->m / kResidentRow + 1 : n + g->m / kExpandArcs + 1;
   const size_t sig_bytes = sizeof(uint64_t) * (size_t)n * pl.Wp;
-  const size_t bm_bytes = sizeof(uint32_t) * (size_t)nbm;
-  const size_t c_bytes = resident ? 2 * bm_bytes : bm_bytes;  // resident: two mark bits a row
   pl.post_wide = !bs && pl.Wp >= kWidePostWords;
-  // the delta buffers keep one all-zero row past the last node (the row a
-  // TMA gather of an empty slot reads)
-  const size_t delta_bytes_alloc = sig_bytes + sizeof(uint64_t) * (size_t)pl.Wp;
-  std::vector<std::pair<DevBuf *, size_t>> needs = {
-      {&w.X, sig_bytes}, {&w.D0, delta_bytes_alloc}, {&w.D1, delta_bytes_alloc},
-      {&w.C0, c_bytes}, {&w.C1, c_bytes}, {&w.Sat, c_bytes},
-      {&w.F0, sizeof(int32_t) * (size_t)n}, {&w.F1, sizeof(int32_t) * (size_t)n},
-      {&w.E, sizeof(unsigned long long) * (size_t)e_cap},
-      {&w.counts, sizeof(uint32_t) * (size_t)row_cap * (size_t)ncols},
-      {&w.rs, sizeof(RoundStats) * (size_t)(row_cap + 2)},
-      {&w.ctrl, sizeof(Ctrl)}, {&w.seeds, sizeof(int32_t) * (size_t)sp}};
-  if (resident) {
-    needs.push_back({&w.F2, sizeof(int32_t) * (size_t)n});
-    needs.push_back({&w.DI, sizeof(uint32_t) * (size_t)n});
-    if (g->out_ptr != g->row_ptr) needs.push_back({&w.DO, sizeof(uint32_t) * (size_t)n});
-  } else {
-    needs.push_back({&w.K0, bm_bytes});
-    needs.push_back({&w.K1, bm_bytes});
-    needs.push_back({&w.A, sizeof(ulonglong2) * (size_t)std::max<int64_t>(npieces, 1)});
-  }
   // one graph's wide rows keep no Y: the pull writes X and D itself
   const bool direct = pl.wide && pl.post_wide;
   if (direct) {  // its post kernel counts in fixed shared memory
     pl.smem_counts = false;
     pl.post_smem = 0;
   }
-  if (!direct) needs.push_back({&w.Y, sig_bytes});
-  if (direct) {
-    needs.push_back({&w.DM0, sizeof(uint32_t) * (size_t)n});
-    needs.push_back({&w.DM1, sizeof(uint32_t) * (size_t)n});
-  } else if (pl.post_wide) {
-    needs.push_back({&w.RB, sizeof(uint32_t) * (size_t)n});
-  }
-  if (pw) {  // claim bits per (word, row); the resident loop: a byte per row
-    const size_t kw = resident ? ((size_t)n + 3) / 4 * 4 : bm_bytes * (size_t)pl.Wp;
-    needs.push_back({&w.KW0, kw});
-    needs.push_back({&w.KW1, kw});
-  }
-  if (bs) needs.push_back({&w.seed_bits, sizeof(int32_t) * (size_t)sp});
   // push rounds (rows of up to 8 words gathered whole): the frontier's
   // out-arc pieces by round parity. The default where they apply: measured
   // faster on the 4096^2 grid by 19%, on R-MAT 22 with s = 256 by 13%, on ER
@@ -1332,17 +1365,11 @@ static pg_status run_pass(Call &cl, const int32_t *seeds_h, int sp, int col0, bo
   // 512-graph mix (batched) by 3%
   const bool push_ok = !pl.wide && pl.CW == pl.Wp;
   const bool push = resident || (push_ok && cl.o.sparse_push != 1);
-  if (push) needs.push_back({&w.E1, sizeof(unsigned long long) * (size_t)e_cap});
-  if (bs && g->nseg > 0) {
-    needs.push_back({&w.gfsum, 3 * sizeof(unsigned long long) * (size_t)g->nseg});
-    needs.push_back({&w.gthr, sizeof(unsigned long long) * (size_t)g->nseg});
-    needs.push_back({&w.dlist, sizeof(int32_t) * (size_t)g->nseg});
-    needs.push_back({&w.dpref, sizeof(int64_t) * ((size_t)g->nseg + 1)});
-  }
   // a packed batch whose caller asked for each graph's m_active: its window
   const bool gm_on = bs && g->nseg > 0 && bs->graph_m && !pw && cl.gm_h;
-  if (gm_on)
-    needs.push_back({&w.gm, sizeof(unsigned long long) * (size_t)(row_cap + 2) * (size_t)g->nseg});
+  const PassShape shape{n, g->m, npieces, g->out_ptr != g->row_ptr, sp, ncols, row_cap,
+                        bs != nullptr, g->nseg, resident, push, pw, gm_on};
+  const WorkspaceNeeds needs = workspace_needs(w, pl, shape);
   if ((rc = carve_workspace(w, needs))) return rc;
   if (!w.ctrl_h) {
     if (cudaMallocHost((void **)&w.ctrl_h, 2 * sizeof(Ctrl)) != cudaSuccess) {
@@ -1811,11 +1838,7 @@ static pg_status propagate(pg_graph *g, const int32_t *seeds, int32_t s, pg_coun
   const int K = s_mode && KW <= 1 ? passes_together(g, npasses, cl.o) : 1;
   const int step = KW > 1 ? 64 * KW : planes;  // seeds per propagation
   const int widest = std::min(step, s);
-  // counts window: up to max_rounds+1 rows, at most ~256 MB of counters
-  int64_t cap_rows = std::max<int64_t>(64, (256LL << 20) / (4LL * widest));
-  if (cl.o.window_rows > 0) cap_rows = cl.o.window_rows;
-  cl.row_cap = (int32_t)std::min<int64_t>((int64_t)out->max_rounds + 1, cap_rows);
-  if (cl.row_cap < 1) cl.row_cap = 1;
+  cl.row_cap = window_rows(widest, out->max_rounds, cl.o);
   pg_stats st{};
   int32_t T = 0, status = PG_OK;
   int passes = 0;
@@ -1858,9 +1881,7 @@ static pg_status propagate(pg_graph *g, const int32_t *seeds, int32_t s, pg_coun
       cr.counts_h = cl.counts_h;
       cr.perm = cl.perm;
       cr.perm_n = cl.perm_n;
-      int64_t rows = std::max<int64_t>(64, (256LL << 20) / (4LL * ns));
-      if (cl.o.window_rows > 0) rows = cl.o.window_rows;
-      cr.row_cap = (int32_t)std::max<int64_t>(1, std::min<int64_t>((int64_t)out->max_rounds + 1, rows));
+      cr.row_cap = window_rows(ns, out->max_rounds, cl.o);
       BatchSeg bs{(const int32_t *)g->rep_graph_of.p, (const int32_t *)g->rep_graph_s.p,
                   (const int32_t *)g->rep_graph_col0.p, bit.data(), ns, planes, gm.data()};
       PassOut po;
@@ -1951,7 +1972,7 @@ static pg_status propagate(pg_graph *g, const int32_t *seeds, int32_t s, pg_coun
   st.sweeps = T + 1;
   st.passes = passes;
   Plan pl;
-  make_plan(g, widest, cl.o, s_mode && KW <= 1, pl);
+  make_plan(g->mean_degree, widest, cl.o, s_mode && KW <= 1, pl);
   st.words_per_row = pl.Wp;
   st.group_lanes = pl.G;
   st.pass_words = KW;
@@ -1995,9 +2016,7 @@ static pg_status propagate_sink(pg_graph *g, const int32_t *seeds, int32_t nseed
   cl.sink_ctx = sink_ctx;
   cl.perm = g->perm_ptr;
   cl.perm_n = g->n;
-  int64_t cap_rows = std::max<int64_t>(64, (256LL << 20) / (4LL * ncols));
-  if (cl.o.window_rows > 0) cap_rows = cl.o.window_rows;
-  cl.row_cap = (int32_t)std::max<int64_t>(1, std::min<int64_t>((int64_t)max_rounds + 1, cap_rows));
+  cl.row_cap = window_rows(ncols, max_rounds, cl.o);
   // each graph's m_active of a packed batch comes from the kernels' window
   const bool per_graph = mact && bs && bs->graph_m && g->nseg > 0;
   std::vector<unsigned long long> gm;
@@ -2043,7 +2062,7 @@ static pg_status propagate_sink(pg_graph *g, const int32_t *seeds, int32_t nseed
   st.post_launches = po.post_launches;
   {
     Plan pl;
-    if (make_plan(g, bs ? bs->s_bits : nseeds, cl.o, false, pl) == PG_OK) {
+    if (make_plan(g->mean_degree, bs ? bs->s_bits : nseeds, cl.o, false, pl) == PG_OK) {
       st.words_per_row = pl.Wp;
       st.group_lanes = pl.G;
       st.pass_words = 1;
@@ -2070,26 +2089,26 @@ pg_status propagate_batch_group(pg_graph *g, const int32_t *seeds, const int32_t
                         st_out, mact);
 }
 
-int64_t workspace_bytes(const pg_graph *g, int32_t s, int32_t max_rounds, int32_t window_rows) {
-  return workspace_bytes_nm(g->n, g->m, s, max_rounds, window_rows);
+int64_t workspace_bytes(const Workspace &w, int64_t n, int64_t m, bool directed, int32_t s,
+                        int32_t ncols, int32_t nseg, int32_t max_rounds, const pg_options &opt) {
+  Plan pl;
+  if (make_plan((double)m / (double)std::max<int64_t>(n, 1), s, opt, false, pl) != PG_OK) return 0;
+  const bool batch = nseg > 0;
+  pl.post_wide = !batch && pl.Wp >= kWidePostWords;
+  const bool narrow = !pl.wide && pl.CW == pl.Wp;
+  const bool resident = narrow && resident_schedule(opt);
+  const PassShape shape{n, m, n + m / (pl.wide ? kWidePiece : 2) + 1, directed, ncols, ncols,
+                        window_rows(ncols, max_rounds, opt), batch, nseg, resident,
+                        resident || (narrow && opt.sparse_push != 1), false, false};
+  const int64_t rctl = resident ? (int64_t)sizeof(ResidentCtl) : 0;
+  return workspace_after(w, workspace_needs(const_cast<Workspace &>(w), pl, shape)) +
+         std::max<int64_t>((int64_t)w.rctl.bytes, rctl);
 }
 
-int64_t workspace_bytes_nm(int64_t n, int64_t m, int32_t s, int32_t max_rounds,
-                           int32_t window_rows) {
-  // the buffers run_pass ensures, sized for the widest plan of s seeds
-  const int W = (s + 63) / 64;
-  const int CW = W <= 1 ? 1 : W <= 2 ? 2 : W <= 4 ? 4 : 8;
-  const int64_t Wp = (W + CW - 1) / CW * CW;
-  const int64_t nbm = (n + 31) / 32;
-  const int64_t pieces = n + m / 2 + 1;  // pieces hold at least 2 arcs
-  const int64_t cap_rows =
-      window_rows > 0 ? window_rows : std::max<int64_t>(64, (256LL << 20) / (4LL * s));
-  const int64_t row_cap = std::max<int64_t>(1, std::min<int64_t>((int64_t)max_rounds + 1, cap_rows));
-  // the frontier's out-arc pieces, twice for push rounds (rows of <= 8 words)
-  const int64_t e_bufs = W <= 8 ? 2 : 1;
-  return 4 * n * Wp * 8 + (5 + 2 * Wp) * nbm * 4 + 3 * n * 4 +
-         e_bufs * (n + m / kExpandArcs + 1) * 8 + pieces * 16 + row_cap * s * 4 + (row_cap + 2) * (int64_t)sizeof(RoundStats) +
-         (int64_t)s * 8 + 4096;
+int64_t piece_list_bytes(int64_t n, int64_t m, int32_t s, const pg_options &opt) {
+  Plan pl;
+  if (make_plan((double)m / (double)std::max<int64_t>(n, 1), s, opt, false, pl) != PG_OK) return 0;
+  return pl.wide ? (n + m / kWidePiece + 1) * (int64_t)sizeof(ulonglong2) : 0;
 }
 
 pg_status propagate_columns(pg_graph *g, const int32_t *seeds, int32_t nseeds, int32_t max_rounds,

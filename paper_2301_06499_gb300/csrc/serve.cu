@@ -157,12 +157,14 @@ int64_t union_array_bytes(int64_t n, int64_t m, bool directed) {
 int64_t slot_need(const pg_server *srv, const Slot &sl, int32_t gid, int32_t s) {
   const pg_graph *g = srv->graphs.at(gid).g;
   const int32_t maxr = (int32_t)std::min<int64_t>(g->n - 1, 0x3FFFFFFF);
-  int64_t ws = std::max(workspace_held(sl.ws),
-                        workspace_bytes(g, s, maxr, srv->cfg.opt.window_rows));
+  const int64_t ws =
+      workspace_bytes(sl.ws, g->n, g->m, g->directed != 0, s, s, 0, maxr, srv->cfg.opt);
   int64_t views = 0;
-  for (const auto &kv : sl.views) views += view_bytes(kv.second);
-  if (!sl.views.count(gid)) views += (g->n + g->m / 2 + 1) * 16;
-  return ws + views;
+  for (const auto &kv : sl.views)
+    if (kv.first != gid) views += view_bytes(kv.second);
+  const auto it = sl.views.find(gid);
+  return ws + views + std::max(it != sl.views.end() ? view_bytes(it->second) : 0,
+                               piece_list_bytes(g->n, g->m, s, srv->cfg.opt));
 }
 
 // Under the lock: the oldest queued request that fits, with the other queued
@@ -223,9 +225,8 @@ bool pick(pg_server *srv, int k, Job &job) {
       if (!uni) return slot_need(srv, me, head->graph, (int32_t)s_total);
       int64_t views = 0;
       for (const auto &kv : me.views) views += view_bytes(kv.second);
-      return std::max(workspace_held(me.ws),
-                      workspace_bytes_nm(un, um, (int32_t)smax, umaxr,
-                                         srv->cfg.opt.window_rows)) +
+      return workspace_bytes(me.ws, un, um, udir, (int32_t)smax, (int32_t)s_total,
+                             (int32_t)per.size(), umaxr, srv->cfg.opt) +
              views + union_array_bytes(un, um, udir);
     };
     int64_t need = need_now();
@@ -723,7 +724,8 @@ pg_status pg_server_submit(pg_server *srv, int32_t graph_id, const int32_t *seed
   // must fit an otherwise idle server
   const int32_t maxr = (int32_t)std::min<int64_t>(g->n - 1, 0x3FFFFFFF);
   const int64_t alone =
-      workspace_bytes(g, s, maxr, srv->cfg.opt.window_rows) + (g->n + g->m / 2 + 1) * 16;
+      workspace_bytes(Workspace{}, g->n, g->m, g->directed != 0, s, s, 0, maxr, srv->cfg.opt) +
+      piece_list_bytes(g->n, g->m, s, srv->cfg.opt);
   if (resident_total(srv) + alone > srv->budget) return PG_ENOMEM;
   r->id = srv->next_req++;
   r->graph = graph_id;

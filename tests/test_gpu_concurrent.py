@@ -101,6 +101,52 @@ def test_two_threads_on_two_graphs():
         raise errors[0]
 
 
+def test_a_batch_beside_calls():
+    """A packed batch whose part of the SMs changes as another thread's calls come
+    and go: its counts windows end at rounds of their own, each graph's m_active
+    among them."""
+    import torch
+    graphs = [I.grid(260, 250, 0.05, 806), I.grid(300, 120, 0.05, 807), I.er(20_000, 6, 808)]
+    seeds = [I.seeds(g.n, 100, 809) for g in graphs]
+    want = [oracle.run(g, x) for g, x in zip(graphs, seeds)]
+    other = I.er(50_000, 8, 810)
+    x = I.seeds(other.n, 64, 811)
+    want_other = oracle.run(other, x)
+    stop, errors = threading.Event(), []
+
+    def calls():
+        try:
+            with torch.cuda.stream(torch.cuda.Stream()), pg.Graph.from_inputs(other) as G:
+                while not stop.is_set():
+                    for _ in range(3):
+                        _check(pg.propagate_p(G, x), want_other)
+                    time.sleep(0.003)
+        except BaseException as e:  # noqa: B902 - the main thread raises it
+            errors.append(e)
+
+    th = threading.Thread(target=calls)
+    th.start()
+    split = False  # the loop ended its launch and went on
+    try:
+        with pg.Batch() as b:
+            for g, sd in zip(graphs, seeds):
+                b.add_inputs(g, sd)
+            for k in range(100):
+                b.set_streams(4 if k == 1 else 1)
+                b.run()
+                for i, w in enumerate(want):
+                    _check(b.result(i), w)
+                split = split or b.stats()["launches"] > b.stats()["groups"]
+                if split and k >= 3:
+                    break
+    finally:
+        stop.set()
+        th.join()
+    if errors:
+        raise errors[0]
+    assert split
+
+
 def test_a_loop_that_ends_after_every_round():
     """Launches of one round each (and so a counts window of one row): pushed and
     swept rounds, passes as words, copies as a packed batch, rows on lane pairs

@@ -118,14 +118,16 @@ typedef struct {
                                (0, the default = the library's choice: 0.2 in
                                the one-launch round loop (use_graphs) for
                                graphs whose rows have at most 64 in-arcs and
-                               0.08 for others, else 0.05) */
+                               0.08 for others, else, and in a packed batch
+                               (of each graph's arcs), 0.05) */
   int32_t group_lanes;      /* lanes sharing one work piece (1..32, power of
                                two); a piece is group_lanes x 8 in-arcs for
                                s <= 128, x 4 for s <= 256, x 2 above, and
                                longer rows are split into
                                pieces combined with atomic OR; 0 = the
                                smallest group whose piece covers the mean
-                               in-degree */
+                               in-degree. Not read by the one-launch round
+                               loop (use_graphs) */
   int32_t test_changed;     /* an in-neighbour u adds to v only the bits u
                                gained in the previous round (its delta, zero
                                if u did not change). 1: test u's changed bit
@@ -140,9 +142,12 @@ typedef struct {
                                without a host round trip: for rows of up to 8
                                words gathered whole (s <= 512, or up to 8
                                passes as words) with sparse_push 0 one
-                               cooperative launch holds the whole round loop,
-                               otherwise a CUDA graph with a device-driven
-                               while node; 0: plain launches in batches */
+                               cooperative launch holds the whole round loop
+                               (launched again where it stopped to share the
+                               device: every 20 ms, and when other calls come
+                               or go), otherwise a CUDA graph with a
+                               device-driven while node; 0: plain launches in
+                               batches */
   int32_t timing;           /* 1: record CUDA events around every kernel
                                launch (plain launches) for pg_last_stats */
   int32_t window_rows;      /* rows of per-round counters kept on the device

@@ -498,8 +498,9 @@ __device__ __forceinline__ int stage_append(const Params &p, Ctrl *ctrl, int32_t
 // kernel (caps registers; the kernels are latency-bound, so occupancy pays:
 // 4 blocks of 256 threads = 64 registers, measured 10% faster than 3 for
 // 4-word rows on R-MAT 22, and 2.6% faster for 8-word rows on the scale-26
-// R-MAT although those spill ~150 bytes at 64 registers) and arcs per lane
-// per step of the dense sweep.
+// R-MAT although those then spilled ~150 bytes at 64 registers; with the early
+// stop's instantiation beside the plain one they spill 310 to 450) and arcs per
+// lane per step of the dense sweep.
 #ifndef PG_PULL_MIN_BLOCKS
 #define PG_PULL_MIN_BLOCKS 4
 #endif
@@ -1102,9 +1103,12 @@ __global__ void __launch_bounds__(kBlock, CW <= 4 ? PG_PULL_MIN_BLOCKS : PG_PULL
 using PullFn = void (*)(Params);
 // The resident round loop (resident.cu): a cooperative launch, counters of up
 // to kResidentCounts columns in shared memory (two rows of them). A block per
-// SM: 512 threads keep 128 registers each (no spills, and twice the gathers in
-// flight per warp) against 1,024 with 64; ER 10^4 178 against 186 us, R-MAT 22
-// 1.87 against 2.05 ms, 1024^2 grid 40.5 against 47.3 ms.
+// SM: 512 threads keep 128 registers each (twice the gathers in flight per warp)
+// against 1,024 with 64; ER 10^4 178 against 186 us, R-MAT 22 1.87 against 2.05
+// ms, 1024^2 grid 40.5 against 47.3 ms. Spills at 128 (stores / loads in bytes):
+// PROPAGATE-S passes of 8 words 56 / 96 (none on lane pairs), of 4 words 32 / 72,
+// of 2 words 8 / 8; packed batches of 2 to 8 words and rows of 8 words whole up
+// to 8 / 4; the others none.
 constexpr int kResidentThreads = 512;
 constexpr int kResidentCounts = 8192;
 constexpr int kResidentSorted = 512;  // most seeds whose bits are placed by degree

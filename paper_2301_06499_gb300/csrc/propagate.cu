@@ -267,8 +267,9 @@ __device__ __forceinline__ void count_wide(const Params &p, const int32_t *F, in
 //     pieces, adding its in-degree to m_active[t+1].
 //  C. last block: fixpoint test (Alg. 1: do ... while Count > 0), hand-over
 //     to round t+1, and, inside a while-graph, the loop condition.
-// Four resident blocks per SM (64 registers, no spills): like the pull, the
-// kernel is latency-bound, and at the default 80 registers only three fit.
+// Four resident blocks per SM (64 registers; WIDE spills 64 bytes of stores and 96
+// of loads, the others nothing): like the pull, the kernel is latency-bound, and
+// at the default 80 registers only three fit.
 //
 // WIDE (rows of 16 or more words, one graph): part A runs over tiles of 32
 // frontier rows x 16 words, so that the grid spreads over the words of a row

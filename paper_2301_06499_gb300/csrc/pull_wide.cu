@@ -35,7 +35,9 @@ namespace pg {
 // of four neighbours are in flight), re-reading the piece's columns (from
 // L1) in each pass.
 // Three resident blocks per SM (80 registers; four of 64 for rows of 32 words):
-// at 88 words four blocks spill, 16.0 against 14.9 ms a call on ER 10^6.
+// at 88 words four blocks spill, 16.0 against 14.9 ms a call on ER 10^6. Three
+// blocks spill too where a lane holds four words (NW = 4, and NW = 0 for rows
+// above 128): about 200 bytes of stores and 120 to 210 of loads.
 //
 // PW: PROPAGATE-S passes as the words of one signature; m_active is counted
 // per pass here, in dense and sparse rounds alike (see count_pass_words).

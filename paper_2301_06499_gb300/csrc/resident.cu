@@ -33,17 +33,20 @@
 // as k_pull does, with its early stop.
 //
 // Measured per call, round by round (with dense rounds that stop early) and
-// here: ER 10^3 (s = 64) 215 -> 90 us, ER 10^4 (s = 64) 288 -> 131 us,
-// 1024^2 grid (s = 128, ~2,050 rounds) 83 -> 36.5 ms, R-MAT 22 (s = 256)
-// 2.23 -> 1.56 ms, R-MAT 26 (s = 512) 54.9 -> 42 ms, 30 packed graphs
-// 33.6 -> 16.3 ms. What bounds it now: a round of little work is five
-// dependent accesses, two block-wide steps and the barrier, 6 to 7 us; heavy
-// pushes the L2's atomics (25 to 28 per ns on spread addresses: the grid sends
-// 0.98 G of them in 34.5 ms), which is why marks are loaded before they are
-// set; heavy sweeps the gathers that a thread's registers hold in flight.
+// here (a range: by the seeds drawn): ER 10^3 (s = 64) 215 -> 94 us, ER 10^4
+// (s = 64) 288 -> 135 us, 1024^2 grid (s = 128, ~2,050 rounds) 83 -> 37.5 ms,
+// R-MAT 22 (s = 256) 2.23 -> 1.5 to 1.7 ms, R-MAT 26 (s = 512) 54.9 -> 43 to
+// 48 ms, 30 packed graphs 33.6 -> 16.4 ms. What bounds it now: a round of
+// little work is five dependent accesses, two block-wide steps and the barrier,
+// 6 to 7 us; heavy pushes the L2's atomics (25 to 28 per ns on spread addresses:
+// the grid sends 0.98 G of them in 34.5 ms), which is why marks are loaded before
+// they are set; heavy sweeps the gathers that a thread's registers hold in
+// flight.
 //
-// Every wait at the barrier is bounded; on expiry the call returns
-// PG_ETIMEOUT. The blocks are co-resident by the cooperative launch.
+// The blocks are co-resident by the cooperative launch. Every wait at the barrier
+// is bounded; on expiry the call returns PG_ETIMEOUT. A launch holds its SMs: it
+// ends early, to go on in another, when other propagations want a part of them
+// and every 20 ms (should_yield, share.cpp).
 #include "kernels.cuh"
 
 namespace pg {
@@ -464,9 +467,10 @@ __device__ __forceinline__ void push_round(const Params &p, Lane &L, const int32
   const int64_t groups = (nF + rows - 1) / rows;
   const unsigned long long *gfp =
       SEG ? p.gfsum + (size_t)((L.t + 2) % 3) * (size_t)p.nseg : nullptr;
-  // a degree is wanted once per claimed row; while all of them sit in L2 it is
-  // fetched with the signature, else after the claim (one access in eight on
-  // the hub rows of R-MAT 26)
+  // a degree is wanted once per claimed row. Up to 2^22 rows (16 MB of degrees,
+  // which stay in L2 beside the signatures a round touches) it is fetched with the
+  // signature, above after the claim: on R-MAT 26 (268 MB of them) one access in
+  // eight on the hub rows. Where between the two it turns was not measured.
   const bool deg_now = p.n <= (1 << 22);
   // row and arcs of an item: fetched for the next item ahead of this one's work
   auto item = [&](int64_t it, int32_t &u, int64_t &ob, int64_t &oe) {

@@ -36,7 +36,7 @@
 // here (a range: by the seeds drawn): ER 10^3 (s = 64) 215 -> 94 us, ER 10^4
 // (s = 64) 288 -> 135 us, 1024^2 grid (s = 128, ~2,050 rounds) 83 -> 37.5 ms,
 // R-MAT 22 (s = 256) 2.23 -> 1.5 to 1.7 ms, R-MAT 26 (s = 512) 54.9 -> 43 to
-// 48 ms, 30 packed graphs 33.6 -> 16.4 ms. What bounds it now: a round of
+// 50 ms, 30 packed graphs 33.6 -> 16.4 ms. What bounds it now: a round of
 // little work is five dependent accesses, two block-wide steps and the barrier,
 // 6 to 7 us; heavy pushes the L2's atomics (25 to 28 per ns on spread addresses:
 // the grid sends 0.98 G of them in 34.5 ms), which is why marks are loaded before

@@ -23,7 +23,7 @@ LIB = os.path.join(OUT_DIR, "libpropagate.so")
 VARIANTS = {"": ("", []),
             # every gather checks its row and word index and records a bad one
             # in the control block instead of faulting (the call returns
-            # PG_EDEVICE); it also exports pg_debug_short_barrier
+            # PG_EDEVICE); it also exports the pg_debug_* calls of the tests
             "debug-bounds": ("_debug_bounds", ["-DPG_DEBUG_BOUNDS"])}
 
 
